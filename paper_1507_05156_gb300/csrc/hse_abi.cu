@@ -447,6 +447,57 @@ struct BatchShape {
 
 int side_slot(int n) { return n == 8 ? 0 : n == 16 ? 1 : n == 18 ? 2 : n == 20 ? 3 : n == 12 ? 4 : -1; }
 
+// Seconds one SM spends on a pair convolution of grid side n: 41 TFLOP/s of 10 N log2 N + 16 N
+// flops on 152 SMs (16^3 and 24^3; only the ratio to the fixed costs below matters).
+double pair_seconds(int n) {
+  const double N = (double)n * n * n;
+  return (10.0 * N * std::log2(N) + 16.0 * N) / 0.27e12;
+}
+
+// Number of ranges the partners (k', j) of an owner tile are split into: the smallest estimated
+// time of list-scheduling `tiles` x ns ranges (partners / ns pairs of t_pair seconds, uneven where
+// ns does not divide, and 4 us an item for its start, owner and result) on `slots` resident CTAs,
+// plus the pass that sums the ranges' outputs (4 us and 3 TB/s over ns outputs).  A finer split
+// must gain 1%.  Beyond 48 waves the last one no longer matters.
+struct SplitChoice {
+  int ns = 1;
+  double seconds = 0.0;
+};
+SplitChoice choose_split(long long tiles, long long partners, double t_pair, long long slots, size_t out_bytes,
+                         int ns_min) {
+  const int ns_cap = (int)std::min<long long>(32, partners);
+  const long long most = 48 * slots;
+  SplitChoice best;
+  best.ns = std::min(ns_min, ns_cap);
+  for (int ns = best.ns; ns <= ns_cap; ++ns) {
+    if (best.seconds > 0.0 && (tiles * ns > most || (size_t)ns * out_bytes > ((size_t)4 << 30))) break;
+    double t = 0.0;
+    if (tiles * ns > most) {
+      t = (double)tiles * ((double)partners * t_pair + ns * 4e-6) / (double)slots;
+    } else {
+      std::map<double, long long> ends{{0.0, slots}};  // end time -> slots that end then
+      for (int sp = 0; sp < ns; ++sp) {
+        const double cost = (double)((sp + 1) * partners / ns - sp * partners / ns) * t_pair + 4e-6;
+        for (long long left = tiles; left > 0;) {  // the items of a range cost the same
+          const auto first = ends.begin();
+          const double end = first->first + cost;
+          const long long take = std::min(left, first->second);
+          if ((first->second -= take) == 0) ends.erase(first);
+          ends[end] += take;
+          left -= take;
+          t = std::max(t, end);
+        }
+      }
+    }
+    if (ns > 1) t += 4e-6 + (double)ns * (double)out_bytes / 3e12;
+    if (best.seconds == 0.0 || t < 0.99 * best.seconds) {
+      best.seconds = t;
+      best.ns = ns;
+    }
+  }
+  return best;
+}
+
 int cuda_fail(cudaError_t e) { return e == cudaSuccess ? HSE_OK : (e == cudaErrorMemoryAllocation ? HSE_ERR_NOMEM : HSE_ERR_CUDA); }
 
 // Every device allocation of a plan goes through here.  Test hook: a plan created while the
@@ -696,8 +747,8 @@ int hse_plan_create(hse_plan* out, const hse_problem* p) {
   HSE_TRY(plan_malloc(plan, &plan->v32, nq * N * sizeof(float)));
   HSE_TRY(plan_malloc(plan, &plan->dv32, nq * N * sizeof(float)));
   if (plan->p.dtype == HSE_C64) {
-    // Split the k' loop so that the work items fill the resident CTA slots in nearly whole
-    // waves; the partial outputs are summed by reduce_splits.
+    // Split the partners so that the work items fill the resident CTA slots evenly; the partial
+    // outputs are summed by reduce_splits.
     int sms = 0;
     HSE_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, plan->device));
     const int occ_blocks = std::max(1, pairconv_c64_occupancy(n1, MODE_APPLY, plan->blocks_per_sm));
@@ -710,27 +761,22 @@ int hse_plan_create(hse_plan* out, const hse_problem* p) {
     size_t buf = 0, comp = 0;
     for (int o = 0; o < 3; ++o) {
       const int T = slots_for(n1);
-      const long long items = (long long)k_own[o] * ((owners[o] + T - 1) / T);
+      const long long partners = (long long)k_part[o] * b_part[o];
       // the staged-partner kernel (roles with owner = target) caches an item's occupations:
       // at most kOccCache partners per item
-      const int ns_cap = std::min(8, k_part[o]);
-      const int ns_min =
-          (plan->blocks_per_sm <= 0 && o != ROLE_OCC)
-              ? std::min(ns_cap, std::max(1, (int)(((long long)k_part[o] * b_part[o] + kOccCache - 1) / kOccCache)))
-              : 1;
-      double best_eff = 0.0;
-      int best = ns_min;
-      for (int ns = ns_min; ns <= ns_cap; ++ns) {
-        const long long it = items * ns;
-        const long long waves = (it + slots - 1) / slots;
-        const double eff = (double)it / (double)(waves * slots);
-        if (eff > best_eff + 0.02) {
-          best_eff = eff;
-          best = ns;
-        }
+      const int ns_min = (plan->blocks_per_sm <= 0 && o != ROLE_OCC)
+                             ? (int)std::min<long long>(8, (partners + kOccCache - 1) / kOccCache)
+                             : 1;
+      const double t_pair = (o == ROLE_OCC ? 2.0 : 1.0) * T * pair_seconds(n1);
+      const size_t out_bytes = o == ROLE_ENERGY ? 0 : (size_t)k_own[o] * owners[o] * N * sizeof(float2);
+      auto tiles = [&](int per) { return (long long)k_own[o] * ((owners[o] + per - 1) / per); };
+      SplitChoice choice = choose_split(tiles(T), partners, t_pair, slots, out_bytes, ns_min);
+      int best = choice.ns;
+      size_t need = (best > 1 && o != ROLE_ENERGY) ? (size_t)best * k_own[o] * owners[o] * N : 0;
+      if (need * sizeof(float2) > ((size_t)4 << 30)) {  // keep split buffers modest
+        best = 1;
+        need = 0;
       }
-      const size_t need = (best > 1 && o != ROLE_ENERGY) ? (size_t)best * k_own[o] * owners[o] * N : 0;
-      if (need * sizeof(float2) > ((size_t)4 << 30)) best = 1;  // keep split buffers modest
       plan->nsplit[o] = best;
       if (best > 1) buf = std::max(buf, need);
       if (o != ROLE_ENERGY) comp = std::max(comp, (size_t)best * k_own[o] * owners[o] * 2 * blocked_stride(n1));
@@ -1069,8 +1115,8 @@ void build_batch(hse_plan plan, int split, void* const* vx_out) {
                       : (q.grid[0] == 12 && bc.layout == 0)                       ? 2
                                                                                   : 0;
     for (int sp = 0; sp < ns; ++sp) {
-      const int kp0 = (int)(((long long)sp * q.nk) / ns), kp1 = (int)(((long long)(sp + 1) * q.nk) / ns);
-      const double cost = (double)(kp1 - kp0) * q.n_occ * n * n * n * std::log2(n);
+      const long long partners = (long long)q.nk * q.n_occ;
+      const double cost = (double)((sp + 1) * partners / ns - sp * partners / ns) * n * n * n * std::log2(n);
       for (int r = 0; r < q.nk * ntiles; ++r) list[which].push_back({cost, {(int)c, sp * q.nk * ntiles + r}});
     }
   }

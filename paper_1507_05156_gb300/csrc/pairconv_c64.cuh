@@ -123,7 +123,7 @@ struct PairArgs {
   int n_own, n_part, n_occ;
   int ntiles;           // ceil(n_own / slots)
   float scale;          // -alpha / (N_k * N): per-pair scale is scale * f
-  int nsplit;           // the k' loop is split into nsplit work items per owner tile
+  int nsplit;           // the partners (k', j) are split into nsplit work items per owner tile
   size_t split_stride;  // elements between the per-split outputs (out: float2, partial: double)
   int* status;          // device status word for failed device-side waits (may be null)
   int inject;           // test hook: 1 = the staged kernel never issues its first partner copy
@@ -142,16 +142,22 @@ struct PairArgs {
   int item_count;       // (0: all items)
 };
 
-// Work item `item` -> (split, k, tile), split slowest: the items of one k' split (one range of
+// Work item `item` -> (split, k, tile), split slowest: the items of one split (one range of
 // partner orbitals) run together, so the partners a wave reads stay in L2 from wave to wave.
+// Split s covers the partners q0 .. q1 - 1 of the list (k', j), j fastest; a range may start and
+// end inside a k'.
 struct ItemIdx {
   int split, k, tile;
+  int q0, q1;
   __device__ __forceinline__ ItemIdx(const PairArgs& a, int item) {
     const int per_split = a.nk_own * a.ntiles;
     split = item / per_split;
     const int rem = item - split * per_split;
     k = rem / a.ntiles;
     tile = rem - k * a.ntiles;
+    const long long partners = (long long)a.nk_part * a.n_part;
+    q0 = (int)(split * partners / a.nsplit);
+    q1 = (int)((split + 1) * partners / a.nsplit);
   }
 };
 
@@ -802,14 +808,14 @@ __device__ __forceinline__ void pairconv_item(const PairArgs& args, int item, fl
   const uint32_t trow0 = tbase + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)((warp >> 2) * GP::COLS_PER_WARP);
   const uint32_t ttab = trow0 + (uint32_t)GP::TAB;
 
-  // work item: (split, k, tile); split s covers partner k-points
-  // [s nk_part / nsplit, (s+1) nk_part / nsplit)
+  // work item: (split, k, tile) and its partners, from kp_begin (band j_begin) to kp_end - 1
+  // (band j_end - 1)
   const ItemIdx it(args, item);
   const int split = it.split;
   const int k = it.k;
   const int band = it.tile * G::T + slot;
-  const int kp_begin = (int)(((long long)split * args.nk_part) / args.nsplit);
-  const int kp_end = (int)(((long long)(split + 1) * args.nk_part) / args.nsplit);
+  const int kp_begin = it.q0 / args.n_part, kp_end = (it.q1 + args.n_part - 1) / args.n_part;
+  const int j_begin = it.q0 - kp_begin * args.n_part, j_end = it.q1 - (kp_end - 1) * args.n_part;
   const bool active = valid && band < args.n_own;
   const int bandc = active ? band : 0;
   const int blk = BLK >= 0 ? BLK : args.blk;
@@ -893,7 +899,7 @@ __device__ __forceinline__ void pairconv_item(const PairArgs& args, int item, fl
       }
     }
   };
-  if (kp_begin == kp_end) fold(true, false, true);  // an empty k' range: zeros
+  if (it.q0 == it.q1) fold(true, false, true);  // no partners: zeros
   const int fspan = fold_span(args.n_part);
 
   // MODE_OCC with the omega gradient fused in: this slot's spectrum scratch and FP64 sum
@@ -901,7 +907,7 @@ __device__ __forceinline__ void pairconv_item(const PairArgs& args, int item, fl
   float2* spec_slot = fuse_w ? spec + (size_t)slot * OrbBlk<n>::NBK : nullptr;
   double wsum = 0.0;
 
-  for (int kp = kp_begin; kp < kp_end; ++kp) {
+  for (int kp = kp_begin; kp < kp_end && it.q0 < it.q1; ++kp) {
     // q = k_i - k_j: APPLY-like modes own i (at k) and pair with j at kp; OCC owns j (at k)
     const int qrow = (MODE == MODE_OCC) ? args.qidx[kp * args.nk_own + k] : args.qidx[k * args.nk_part + kp];
     const float* dvrow = fuse_w ? args.vtab2 + (size_t)qrow * G::N : nullptr;
@@ -911,7 +917,8 @@ __device__ __forceinline__ void pairconv_item(const PairArgs& args, int item, fl
       else
         cache_kernel_row<n, PPT, false, n * n, TS>(t, ttab, args.vtab + (size_t)qrow * G::N, args.scale);
     }
-    for (int j = 0; j < args.n_part; ++j) {
+    const int j1 = kp == kp_end - 1 ? j_end : args.n_part;
+    for (int j = kp == kp_begin ? j_begin : 0; j < j1; ++j) {
       const float2* part = args.part + ((size_t)kp * args.n_part + j) * ostr;
       if constexpr (MODE != MODE_OCC) {
         const float f = (float)args.occ[kp * args.n_occ + j];

@@ -182,17 +182,19 @@ struct LayoutOne : LayoutLin<n, 1> {};
 // Occupations of one work item's partners, cached in shared memory when they fit.
 constexpr int kOccCache = 1024;
 
-// Occupation of partner q of the item (q = (kp - kp_begin) * n_part + j): from the shared
+// Occupation of partner q of the item (partner q0 + q of the list (k', j)): from the shared
 // cache, or from global memory past its end.
-__device__ __forceinline__ float item_occ(const float* occ_sh, const PairArgs& a, int kp_begin, int q) {
-  if (q < kOccCache) return occ_sh[q];
-  const int kp = kp_begin + q / a.n_part, j = q - (q / a.n_part) * a.n_part;
-  return (float)a.occ[kp * a.n_occ + j];
+__device__ __forceinline__ float partner_occ(const PairArgs& a, int q) {
+  const int kp = q / a.n_part;
+  return (float)a.occ[kp * a.n_occ + (q - kp * a.n_part)];
+}
+__device__ __forceinline__ float item_occ(const float* occ_sh, const PairArgs& a, int q0, int q) {
+  return q < kOccCache ? occ_sh[q] : partner_occ(a, q0 + q);
 }
 
 // Next partner index q' >= q with nonzero occupation.
-__device__ __forceinline__ int next_partner(const float* occ_sh, const PairArgs& a, int kp_begin, int q, int npairs) {
-  while (q < npairs && item_occ(occ_sh, a, kp_begin, q) == 0.f) ++q;
+__device__ __forceinline__ int next_partner(const float* occ_sh, const PairArgs& a, int q0, int q, int npairs) {
+  while (q < npairs && item_occ(occ_sh, a, q0, q) == 0.f) ++q;
   return q;
 }
 
@@ -238,16 +240,13 @@ __device__ __forceinline__ bool staged_item(const PairArgs& args, const CUtensor
   const int band = it.tile * G::T + slot;
   const bool active = valid && band < args.n_own;
   const int bandc = active ? band : 0;
-  const int kp_begin = (int)(((long long)split * args.nk_part) / args.nsplit);
-  const int kp_end = (int)(((long long)(split + 1) * args.nk_part) / args.nsplit);
-  const int npairs = (kp_end - kp_begin) * args.n_part;
+  const int q0 = it.q0, npairs = it.q1 - it.q0, kp_begin = it.q0 / args.n_part;
   const float2* own = args.own + ((size_t)k * args.n_own + bandc) * G::N;
 
   // fill stage buffer `buf` with partner q (warp 0 only)
   auto fill = [&](int q, int buf) {
     if (lane == 0) {
-      const int kp = kp_begin + q / args.n_part, j = q - (q / args.n_part) * args.n_part;
-      const int row0 = (kp * args.n_part + j) * G::NN;
+      const int row0 = (q0 + q) * G::NN;
       float2* dst = stage + buf * S::STAGE_CPX;
       mbar_arrive_expect_tx(&sh.mbar[buf], (uint32_t)S::STAGE_TX);
 #pragma unroll
@@ -257,12 +256,9 @@ __device__ __forceinline__ bool staged_item(const PairArgs& args, const CUtensor
   };
 
   // the item's partner occupations, once (work items are sized so that they fit)
-  for (int i = tid; i < npairs && i < kOccCache; i += blockDim.x) {
-    const int kp = kp_begin + i / args.n_part, j = i - (i / args.n_part) * args.n_part;
-    sh.occ[i] = (float)args.occ[kp * args.n_occ + j];
-  }
+  for (int i = tid; i < npairs && i < kOccCache; i += blockDim.x) sh.occ[i] = partner_occ(args, q0 + i);
   __syncthreads();
-  int q = next_partner(sh.occ, args, kp_begin, 0, npairs);
+  int q = next_partner(sh.occ, args, q0, 0, npairs);
   if (warp == 0 && q < npairs && args.inject != 1 && !sh.abort) {
     fence_proxy_async_smem();  // earlier generic accesses to this shared memory come first
     fill(q, 0);
@@ -335,8 +331,8 @@ __device__ __forceinline__ bool staged_item(const PairArgs& args, const CUtensor
   int buf = 0;
   int cur_kp = -1;
   while (q < npairs) {
-    const int kp = kp_begin + q / args.n_part;
-    const float f = item_occ(sh.occ, args, kp_begin, q);
+    const int kp = (q0 + q) / args.n_part;
+    const float f = item_occ(sh.occ, args, q0, q);
     if (kp != cur_kp) {
       // a new fold group (fold_span k-points) starts: fold the previous one
       if (cur_kp >= 0 && (kp - kp_begin) / fspan != (cur_kp - kp_begin) / fspan) fold(false);
@@ -354,7 +350,7 @@ __device__ __forceinline__ bool staged_item(const PairArgs& args, const CUtensor
     }
     if (buf) phase1 ^= 1u; else phase0 ^= 1u;
     const float2* stg = stage + buf * S::STAGE_CPX;
-    const int qn = next_partner(sh.occ, args, kp_begin, q + 1, npairs);
+    const int qn = next_partner(sh.occ, args, q0, q + 1, npairs);
     // refill stage[buf ^ 1] with the next partner once every thread is past its last read of it
     // (the previous pair's Z inverse)
     auto refill = [&]() {
