@@ -9,6 +9,8 @@ import sys
 
 WIDTHS = (4, 6, 8, 10, 12, 16, 18, 20, 24, 32, 36, 40, 48)  # n or 2n floats of one pencil, n in {4..24} even
 
+SPLIT = (16, 32)  # widths of the split (issue / wait / put) helpers
+
 
 def chunks(w):
     out, col = [], 0
@@ -59,6 +61,51 @@ def gen_store(w):
     return "\n".join(lines)
 
 
+def gen_issue(w):
+    """Load without its wait: the registers are valid after tmem_wait_ld on them."""
+    lines = [f"__device__ __forceinline__ void tmem_issue_row{w}(uint32_t taddr, float* v) {{"]
+    body, reg = [], 0
+    cs = chunks(w)
+    for ci, (col, c) in enumerate(cs):
+        regs = ", ".join(f"%{reg + i}" for i in range(c))
+        sep = "\\n\\t" if ci + 1 < len(cs) else ""
+        body.append(f'"tcgen05.ld.sync.aligned.32x32b.x{c}.b32 {{{regs}}}, [%{w + ci}];{sep}"')
+        reg += c
+    outs = ", ".join(f'"=f"(v[{i}])' for i in range(w))
+    addrs = ", ".join(f'"r"(taddr + {col}u)' for col, _ in cs)
+    lines.append("  asm volatile(" + "\n               ".join(body))
+    lines.append(f"               : {outs}")
+    lines.append(f"               : {addrs});")
+    lines.append("}")
+    return "\n".join(lines)
+
+
+def gen_wait(w):
+    lines = [f"__device__ __forceinline__ void tmem_wait_ld{w}(float* v) {{"]
+    outs = ", ".join(f'"+f"(v[{i}])' for i in range(w))
+    lines.append(f'  asm volatile("tcgen05.wait::ld.sync.aligned;" : {outs});')
+    lines.append("}")
+    return "\n".join(lines)
+
+
+def gen_put(w):
+    """Store without its wait and without a memory clobber (see tmem_wait_st)."""
+    lines = [f"__device__ __forceinline__ void tmem_put_row{w}(uint32_t taddr, const float* v) {{"]
+    cs = chunks(w)
+    body, reg = [], len(cs)
+    for ci, (col, c) in enumerate(cs):
+        regs = ", ".join(f"%{reg + i}" for i in range(c))
+        sep = "\\n\\t" if ci + 1 < len(cs) else ""
+        body.append(f'"tcgen05.st.sync.aligned.32x32b.x{c}.b32 [%{ci}], {{{regs}}};{sep}"')
+        reg += c
+    ins = ", ".join(f'"f"(v[{i}])' for i in range(w))
+    addrs = ", ".join(f'"r"(taddr + {col}u)' for col, _ in cs)
+    lines.append("  asm volatile(" + "\n               ".join(body))
+    lines.append(f"               :: {addrs}, {ins});")
+    lines.append("}")
+    return "\n".join(lines)
+
+
 def main():
     out = ["// tmem_gen.cuh - generated by gen_tmem.py; do not edit.",
            "// Row helpers: W consecutive 32-bit TMEM columns of this thread's lane, one wait each.",
@@ -68,6 +115,15 @@ def main():
         out.append("")
         out.append(gen_store(w))
         out.append("")
+    out.append("// Split helpers, for pipelines that overlap TMEM traffic with other work: issue, wait (on the")
+    out.append("// same registers), put and one wait for several puts.  No memory clobber: TMEM is not memory")
+    out.append("// the compiler knows, and shared-memory accesses may move across them.")
+    for w in SPLIT:
+        for g in (gen_issue, gen_wait, gen_put):
+            out.append(g(w))
+            out.append("")
+    out.append("__device__ __forceinline__ void tmem_wait_st() { asm volatile(\"tcgen05.wait::st.sync.aligned;\"); }")
+    out.append("")
     out.append("template <int W> struct TmemRow;")
     for w in WIDTHS:
         out.append(f"template <> struct TmemRow<{w}> {{")

@@ -109,7 +109,8 @@ static std::atomic<uint64_t> g_launches{0};
 constexpr int kMaxBatchSplit = 4;
 
 // The CUDA driver API's tensor-map encoder, obtained through the runtime (no link against libcuda).
-cudaError_t make_partner_tmap(CUtensorMap* map, const void* base, int n, long long rows, int sp, int box_rows) {
+cudaError_t make_partner_tmap(CUtensorMap* map, const void* base, int n, long long rows, int sp, int box_rows,
+                              bool swizzle) {
   static PFN_cuTensorMapEncodeTiled_v12000 encode = nullptr;
   if (!encode) {
     void* fn = nullptr;
@@ -125,7 +126,8 @@ cudaError_t make_partner_tmap(CUtensorMap* map, const void* base, int n, long lo
   const cuuint32_t box[2] = {(cuuint32_t)(2 * sp), (cuuint32_t)box_rows};
   const cuuint32_t estr[2] = {1, 1};
   const CUresult r = encode(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, const_cast<void*>(base), dims, strides, box, estr,
-                            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+                            CU_TENSOR_MAP_INTERLEAVE_NONE,
+                            swizzle ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_NONE,
                             CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
@@ -286,6 +288,7 @@ struct hse_plan_s {
   bool blocked = true;       // pencil-load launches read pencil-blocked copies (HSE_PENCIL_BLOCKS=0: no)
   int blocks_per_sm = 0;     // fused-kernel variant: 0 default, -1/-2 staged-partner layouts, 1/2/3/5 pencil loads,
                              // kTcVariant the tensor-core form (HSE_C64_TC)
+  bool wide = false;         // the apply runs the two-exchange 16^3 kernel (kWideVariant)
   bool tc = false;           // created as HSE_C64_TC (p.dtype then reads HSE_C64)
   int inject = 0;            // test hook (HSE_INJECT_SKIP_FILL=1 at plan creation)
   long long alloc_count = 0;   // device allocations made by this plan so far (plan_malloc)
@@ -453,6 +456,7 @@ double pair_seconds(int n) {
   const double N = (double)n * n * n;
   return (10.0 * N * std::log2(N) + 16.0 * N) / 0.27e12;
 }
+constexpr double kWidePairSeconds = 7.1e-6;  // one partner of a tile of the two-exchange 16^3 kernel
 
 // Number of ranges the partners (k', j) of an owner tile are split into: the smallest estimated
 // time of list-scheduling `tiles` x ns ranges (partners / ns pairs of t_pair seconds, uneven where
@@ -691,6 +695,7 @@ int hse_plan_create(hse_plan* out, const hse_problem* p) {
   if (const char* env = std::getenv("HSE_BLOCKS_PER_SM")) {
     const int v = std::atoi(env);
     plan->blocks_per_sm = (v < -2 || v > kOneVariant || v == kTcVariant) ? 0 : v;
+    plan->wide = v == kWideVariant && p->dtype == HSE_C64 && p->grid[0] == 16;  // also where it is slower
   }
   if (plan->tc) plan->blocks_per_sm = kTcVariant;
   const int n1 = p->grid[0], n2 = p->grid[1], n3 = p->grid[2];
@@ -771,6 +776,11 @@ int hse_plan_create(hse_plan* out, const hse_problem* p) {
       const size_t out_bytes = o == ROLE_ENERGY ? 0 : (size_t)k_own[o] * owners[o] * N * sizeof(float2);
       auto tiles = [&](int per) { return (long long)k_own[o] * ((owners[o] + per - 1) / per); };
       SplitChoice choice = choose_split(tiles(T), partners, t_pair, slots, out_bytes, ns_min);
+      if (o == ROLE_TGT && n1 == 16 && plan->blocks_per_sm == 0) {
+        const SplitChoice wide = choose_split(tiles(kWideSlots), partners, kWidePairSeconds, sms, out_bytes, ns_min);
+        plan->wide = plan->wide || wide.seconds < choice.seconds;
+        if (plan->wide) choice = wide;
+      }
       int best = choice.ns;
       size_t need = (best > 1 && o != ROLE_ENERGY) ? (size_t)best * k_own[o] * owners[o] * N : 0;
       if (need * sizeof(float2) > ((size_t)4 << 30)) {  // keep split buffers modest
@@ -849,7 +859,7 @@ int hse_plan_create(hse_plan* out, const hse_problem* p) {
                  plan->nsplit[ROLE_TGT], plan->nsplit[ROLE_ENERGY], plan->nsplit[ROLE_OCC],
                  !c64 ? "staged FP64" : (pairconv_c64_pencil_load(n1, MODE_APPLY, plan->blocks_per_sm)
                                              ? (plan->tc ? "pencil-load, tensor-core Y/X" : "pencil-load")
-                                                                                                    : "staged-partner"),
+                                             : plan->wide ? "two-exchange" : "staged-partner"),
                  plan->blocked ? "on" : "off");
   }
   *out = plan;
@@ -938,7 +948,8 @@ int to_blocked(hse_plan plan, int mode, PairArgs& a, cudaStream_t st) {
 
 int run_pairconv(hse_plan plan, int mode, PairArgs a, int n_own, cudaStream_t st) {
   const int n = plan->p.grid[0];
-  const int T = slots_for(n);
+  const int variant = mode == MODE_APPLY && plan->wide ? kWideVariant : plan->blocks_per_sm;
+  const int T = owner_slots(n, variant);
   a.n_own = n_own;
   if (pairconv_c64_pencil_load(n, mode, plan->blocks_per_sm) && plan->blocked) {
     const int rc = to_blocked(plan, mode, a, st);
@@ -983,10 +994,10 @@ int run_pairconv(hse_plan plan, int mode, PairArgs a, int n_own, cudaStream_t st
     for (long long c0 = 0; c0 < items && e == cudaSuccess; c0 += kSpecCtas) {
       a.item0 = (int)c0;
       a.item_count = (int)std::min<long long>(kSpecCtas, items - c0);
-      e = launch_pairconv_c64(n, mode, a, plan->blocks_per_sm, st);
+      e = launch_pairconv_c64(n, mode, a, variant, st);
     }
   } else {
-    e = launch_pairconv_c64(n, mode, a, plan->blocks_per_sm, st);
+    e = launch_pairconv_c64(n, mode, a, variant, st);
   }
   if (e != cudaSuccess) return cuda_fail(e);
   if ((mode == MODE_APPLY || mode == MODE_OCC) && a.nsplit > 1) {

@@ -199,7 +199,21 @@ constexpr bool pencil_one_fits() {
 
 // Staged-partner kernel (pairconv_tma.cuh): one CTA per SM.
 // Encodes the tensor map of a partner array for the staged-partner kernel of side n.
-cudaError_t make_partner_tmap(CUtensorMap* map, const void* base, int n, long long rows, int sp, int box_rows);
+// swizzle: the 128-byte TMA swizzle (rows of exactly 128 bytes) instead of a padded pitch.
+cudaError_t make_partner_tmap(CUtensorMap* map, const void* base, int n, long long rows, int sp, int box_rows,
+                              bool swizzle = false);
+
+// Two-exchange kernel of the 16^3 apply (kWideVariant, pairconv_wide.cuh): four owners a CTA.  A
+// pair of its tile takes 7.1 us however few of the four slots are filled (two warps a scheduler
+// that mostly wait for themselves), a pair of the staged kernel's two-owner tile 4.1 us; so it is
+// for plans with enough tiles, which choose it by estimated time (hse_plan_create): 12^3
+// k-points, 4^3 sampled, 16 bands 386 -> 317 ms, 3^3 k, 8 bands 690 -> 590 us, but 4 x 2 k, 6 bands
+// 73 us against 55 us staged.
+constexpr int kWideVariant = 6;
+constexpr int kWideSlots = 4;
+cudaError_t launch_pairconv_wide16(const PairArgs& args, cudaStream_t stream);
+// owner orbitals per work item of the kernel that (n, variant) runs
+constexpr int owner_slots(int n, int variant) { return variant == kWideVariant ? kWideSlots : slots_for(n); }
 
 template <int n, int MODE, template <int> class L>
 cudaError_t launch_pairconv_tma(const PairArgs& args, cudaStream_t stream) {
@@ -240,7 +254,8 @@ constexpr bool tma_fits() {
 // 1 or 2 the pencil-load kernel with that occupancy; 3 the ragged pencil-load kernel
 // (pencil_ragged_fits; 24^3 99.6 -> 95.6 ms on the 4x4x4 k, 16-band cell against two pencils a
 // thread on 9 warps); 4 (kTcVariant) its tensor-core form where tc_fits, else the ragged
-// kernel; 5 (kOneVariant) the one-pencil pencil-load kernel where pencil_one_fits.
+// kernel; 5 (kOneVariant) the one-pencil pencil-load kernel where pencil_one_fits; 6
+// (kWideVariant) the two-exchange kernel (16^3 apply only; chosen by the plan).
 // A variant that does not exist for the size falls back to the default.
 template <int n, int MODE>
 constexpr int staged_layout(int variant) {
@@ -254,6 +269,9 @@ constexpr int staged_layout(int variant) {
 
 template <int n, int MODE>
 cudaError_t launch_pairconv_mode(const PairArgs& args, int variant, cudaStream_t stream) {
+  if constexpr (n == 16 && MODE == MODE_APPLY) {
+    if (variant == kWideVariant) return launch_pairconv_wide16(args, stream);
+  }
   switch (staged_layout<n, MODE>(variant)) {
     case -1:
       if constexpr (tma_fits<n, MODE, LayoutSeq>()) return launch_pairconv_tma<n, MODE, LayoutSeq>(args, stream);
