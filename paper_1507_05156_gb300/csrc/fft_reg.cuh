@@ -148,29 +148,120 @@ struct Butterfly<4, DIR, T> {
   }
 };
 
+// 32 operations: the cosine sums through t1 + t2 and t1 - t2 (c1 + c2 = -1/2, c1 - c2 = sqrt(5)/2),
+// the sine sums as s1 (t3 + r t4) and s1 (r t3 - t4), r = s2 / s1, with the factor s1 in the last
+// multiply-adds (36 with the four products written out).
 template <int DIR, typename T>
 struct Butterfly<5, DIR, T> {
   static __host__ __device__ __forceinline__ void run(cpx<T>* a) {
-    constexpr T c1 = T(trig2pi(1, 5, 0));
-    constexpr T c2 = T(trig2pi(2, 5, 0));
+    constexpr T hr5 = T(0.559016994374947424102293417182819059);  // sqrt(5) / 4
     constexpr T s1 = T(DIR * trig2pi(1, 5, 1));
-    constexpr T s2 = T(DIR * trig2pi(2, 5, 1));
+    constexpr T r = T(trig2pi(2, 5, 1) / trig2pi(1, 5, 1));
     const cpx<T> t1 = cadd(a[1], a[4]);
     const cpx<T> t2 = cadd(a[2], a[3]);
     const cpx<T> t3 = csub(a[1], a[4]);
     const cpx<T> t4 = csub(a[2], a[3]);
-    const cpx<T> p1 = {a[0].x + c1 * t1.x + c2 * t2.x, a[0].y + c1 * t1.y + c2 * t2.y};
-    const cpx<T> p2 = {a[0].x + c2 * t1.x + c1 * t2.x, a[0].y + c2 * t1.y + c1 * t2.y};
-    // i (s1 t3 + s2 t4) and i (s2 t3 - s1 t4)
-    const cpx<T> q1 = {-(s1 * t3.y + s2 * t4.y), s1 * t3.x + s2 * t4.x};
-    const cpx<T> q2 = {-(s2 * t3.y - s1 * t4.y), s2 * t3.x - s1 * t4.x};
-    a[0] = {a[0].x + t1.x + t2.x, a[0].y + t1.y + t2.y};
-    a[1] = cadd(p1, q1);
-    a[4] = csub(p1, q1);
-    a[2] = cadd(p2, q2);
-    a[3] = csub(p2, q2);
+    const cpx<T> t = cadd(t1, t2), u = csub(t1, t2);
+    const cpx<T> m = {a[0].x - T(0.25) * t.x, a[0].y - T(0.25) * t.y};
+    const cpx<T> p1 = {m.x + hr5 * u.x, m.y + hr5 * u.y};
+    const cpx<T> p2 = {m.x - hr5 * u.x, m.y - hr5 * u.y};
+    const cpx<T> q1 = {t3.x + r * t4.x, t3.y + r * t4.y};
+    const cpx<T> q2 = {r * t3.x - t4.x, r * t3.y - t4.y};
+    a[0] = cadd(a[0], t);
+    a[1] = {p1.x - s1 * q1.y, p1.y + s1 * q1.x};
+    a[4] = {p1.x + s1 * q1.y, p1.y - s1 * q1.x};
+    a[2] = {p2.x - s1 * q2.y, p2.y + s1 * q2.x};
+    a[3] = {p2.x + s1 * q2.y, p2.y - s1 * q2.x};
   }
 };
+
+// Last butterfly of a 4-point column whose twiddles are folded in: s0, s1 are the sum and the
+// difference of the even inputs, the odd inputs are c u1 and c u3 with one real c, which rides on
+// the multiply-adds.
+template <int DIR, typename T>
+__host__ __device__ __forceinline__ void fold_column(cpx<T>* a, cpx<T> s0, cpx<T> s1, cpx<T> u1, cpx<T> u3, T c) {
+  const cpx<T> t0 = cadd(u1, u3), t1 = mul_i<DIR>(csub(u1, u3));
+  a[0] = {s0.x + c * t0.x, s0.y + c * t0.y};
+  a[2] = {s0.x - c * t0.x, s0.y - c * t0.y};
+  a[1] = {s1.x + c * t1.x, s1.y + c * t1.y};
+  a[3] = {s1.x - c * t1.x, s1.y - c * t1.y};
+}
+// x (1 + DIR i t) and x (t + DIR i)
+template <int DIR, typename T>
+__host__ __device__ __forceinline__ cpx<T> mul_1t(cpx<T> x, T t) {
+  const T s = DIR * t;
+  return {x.x - s * x.y, x.y + s * x.x};
+}
+template <int DIR, typename T>
+__host__ __device__ __forceinline__ cpx<T> mul_t1(cpx<T> x, T t) {
+  if constexpr (DIR > 0) return {t * x.x - x.y, t * x.y + x.x};
+  else return {t * x.x + x.y, t * x.y - x.x};
+}
+// x (1 + DIR i) and x (DIR i - 1)
+template <int DIR, typename T>
+__host__ __device__ __forceinline__ cpx<T> mul_11(cpx<T> x) {
+  if constexpr (DIR > 0) return {x.x - x.y, x.y + x.x};
+  else return {x.x + x.y, x.y - x.x};
+}
+template <int DIR, typename T>
+__host__ __device__ __forceinline__ cpx<T> mul_i1(cpx<T> x) {
+  if constexpr (DIR > 0) return {-x.x - x.y, x.x - x.y};
+  else return {x.y - x.x, -x.x - x.y};
+}
+
+// 8 and 16 points, 4-point columns with folded twiddles: 52 and 144 operations instead of 56 and
+// 164 with a complex multiplication per twiddle.
+template <int DIR, typename T>
+__host__ __device__ __forceinline__ void fft8_fold(cpx<T>* a) {
+  constexpr T h = T(trig2pi(1, 8, 0));
+  cpx<T> s[4], d[4];
+  static_for<0, 4>([&](auto rc) {
+    constexpr int r = decltype(rc)::value;
+    s[r] = cadd(a[r], a[r + 4]);
+    d[r] = csub(a[r], a[r + 4]);
+  });
+  Butterfly<4, DIR, T>::run(s);
+  cpx<T> o[4];
+  const cpx<T> e = mul_i<DIR>(d[2]);
+  fold_column<DIR, T>(o, cadd(d[0], e), csub(d[0], e), mul_11<DIR, T>(d[1]), mul_i1<DIR, T>(d[3]), h);
+  static_for<0, 4>([&](auto kc) {
+    constexpr int k = decltype(kc)::value;
+    a[2 * k] = s[k];
+    a[2 * k + 1] = o[k];
+  });
+}
+
+template <int DIR, typename T>
+__host__ __device__ __forceinline__ void fft16_fold(cpx<T>* a) {
+  constexpr T h = T(trig2pi(2, 16, 0)), c1 = T(trig2pi(1, 16, 0));
+  constexpr T t = T(trig2pi(1, 16, 1) / trig2pi(1, 16, 0));
+  cpx<T> m[4][4];  // m[k][r]: output k of the DFT over a[r], a[4 + r], a[8 + r], a[12 + r]
+  static_for<0, 4>([&](auto rc) {
+    constexpr int r = decltype(rc)::value;
+    cpx<T> c[4] = {a[r], a[4 + r], a[8 + r], a[12 + r]};
+    Butterfly<4, DIR, T>::run(c);
+    static_for<0, 4>([&](auto kc) { m[decltype(kc)::value][r] = c[decltype(kc)::value]; });
+  });
+  Butterfly<4, DIR, T>::run(m[0]);
+  {  // W = c1 (1 +- i t), W^2 = h (1 +- i), W^3 = c1 (t +- i)
+    const cpx<T> u = mul_11<DIR, T>(m[1][2]);
+    fold_column<DIR, T>(m[1], {m[1][0].x + h * u.x, m[1][0].y + h * u.y}, {m[1][0].x - h * u.x, m[1][0].y - h * u.y},
+                        mul_1t<DIR, T>(m[1][1], t), mul_t1<DIR, T>(m[1][3], t), c1);
+  }
+  {  // W^2, W^4 = +- i, W^6 = h (+- i - 1)
+    const cpx<T> u = mul_i<DIR>(m[2][2]);
+    fold_column<DIR, T>(m[2], cadd(m[2][0], u), csub(m[2][0], u), mul_11<DIR, T>(m[2][1]), mul_i1<DIR, T>(m[2][3]), h);
+  }
+  {  // W^3, W^6, W^9 = -c1 (1 +- i t)
+    const cpx<T> u = mul_i1<DIR, T>(m[3][2]);
+    const cpx<T> w = mul_1t<DIR, T>(m[3][3], t);
+    fold_column<DIR, T>(m[3], {m[3][0].x + h * u.x, m[3][0].y + h * u.y}, {m[3][0].x - h * u.x, m[3][0].y - h * u.y},
+                        mul_t1<DIR, T>(m[3][1], t), {-w.x, -w.y}, c1);
+  }
+  static_for<0, 4>([&](auto kc) {
+    static_for<0, 4>([&](auto sc) { a[decltype(kc)::value + 4 * decltype(sc)::value] = m[decltype(kc)::value][decltype(sc)::value]; });
+  });
+}
 
 __host__ __device__ constexpr int pick_radix(int n) {
   return (n % 4 == 0) ? 4 : (n % 2 == 0) ? 2 : (n % 3 == 0) ? 3 : (n % 5 == 0) ? 5 : n;
@@ -208,12 +299,17 @@ __host__ __device__ constexpr int crt_index(int k1, int k2, int n1, int n2) {
 template <int N, int DIR, typename T>
 __host__ __device__ __forceinline__ void fft(cpx<T>* a);
 
-// Cooley-Tukey (decimation in time) for prime powers: N = R * M with twiddles.
-template <int N, int DIR, typename T>
+// Cooley-Tukey (decimation in time) for prime powers: N = R * M with twiddles (FOLD: the folded
+// forms of 8 and 16).
+template <int N, int DIR, typename T, bool FOLD = true>
 __host__ __device__ __forceinline__ void fft_ct(cpx<T>* a) {
   constexpr int R = pick_radix(N);
   if constexpr (R == N) {
     Butterfly<N, DIR, T>::run(a);
+  } else if constexpr (FOLD && N == 8) {
+    fft8_fold<DIR, T>(a);
+  } else if constexpr (FOLD && N == 16) {
+    fft16_fold<DIR, T>(a);
   } else {
     constexpr int M = N / R;
     cpx<T> sub[R][M];
@@ -260,7 +356,10 @@ __host__ __device__ __forceinline__ void fft_pfa(cpx<T>* a) {
     constexpr int k2 = decltype(c2)::value;
     cpx<T> col[N1];
     static_for<0, N1>([&](auto c1) { col[decltype(c1)::value] = m[decltype(c1)::value][k2]; });
-    fft<N1, DIR, T>(col);
+    // FP32 24 points: the 24^3 kernel has no registers to spare for the folded 8-point form
+    // (24^3, 64 k, 32 sampled, 16 + 32 bands: 51.2 -> 52.1 ms with it)
+    if constexpr (N1 == 8 && sizeof(T) == 4) fft_ct<N1, DIR, T, false>(col);
+    else fft<N1, DIR, T>(col);
     static_for<0, N1>([&](auto c1) {
       constexpr int k1 = decltype(c1)::value;
       constexpr int k = crt_index(k1, k2, N1, N2);
