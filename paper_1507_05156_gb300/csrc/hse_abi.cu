@@ -31,6 +31,7 @@
 #include <nvtx3/nvToolsExt.h>
 
 #include "../../include/hse_fock.h"
+#include "fused_f64.cuh"
 #include "launch.cuh"
 
 namespace hse {
@@ -102,6 +103,19 @@ __global__ void reduce_splits(float4* __restrict__ out, const float4* __restrict
     float4 a = buf[i], c = make_float4(0.f, 0.f, 0.f, 0.f);
     for (int sp = 1; sp < nsplit; ++sp) fold4(a, c, buf[(size_t)sp * count4 + i], c);
     out[i] = make_float4(a.x + c.x, a.y + c.y, a.z + c.z, a.w + c.w);
+  }
+}
+
+// The same for complex128 (plain sums, splits in ascending order).
+__global__ void reduce_splits_f64(double2* __restrict__ out, const double2* __restrict__ buf, int nsplit, size_t count) {
+  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < count; i += (size_t)gridDim.x * blockDim.x) {
+    double2 s = buf[i];
+    for (int sp = 1; sp < nsplit; ++sp) {
+      const double2 c = buf[(size_t)sp * count + i];
+      s.x += c.x;
+      s.y += c.y;
+    }
+    out[i] = s;
   }
 }
 
@@ -281,8 +295,12 @@ struct hse_plan_s {
   float* dv32 = nullptr;
   double* partial = nullptr; // device [nk * max(n_occ, n_tgt)]
   int* status = nullptr;     // device status word
-  // complex128 staged form
-  double2* work = nullptr;   // [batch][N]
+  // complex128, per OwnerRole: the fused kernel (where the grid fits shared memory and the schedule
+  // is estimated shorter) with its tile size and split, or the staged form
+  bool fused64[3] = {false, false, false};
+  int f64_T[3] = {1, 1, 1}, f64_ns[3] = {1, 1, 1};
+  double2* split64 = nullptr;  // [nsplit][owners][N] partial outputs when a role's nsplit > 1
+  double2* work = nullptr;   // staged: [batch][N]
   size_t work_pairs = 0;
   double2* vx64 = nullptr;   // [nk][max(n_occ, n_tgt)][N]
   bool blocked = true;       // pencil-load launches read pencil-blocked copies (HSE_PENCIL_BLOCKS=0: no)
@@ -456,19 +474,42 @@ double pair_seconds(int n) {
   const double N = (double)n * n * n;
   return (10.0 * N * std::log2(N) + 16.0 * N) / 0.27e12;
 }
+// The fused FP64 kernel with T orbitals a CTA: CTAs an SM holds, seconds of its FP64 pipe a partner
+// takes (about 8 GFLOP/s of the same count, a partial warp costing a whole one), and seconds a
+// partner takes in a CTA that has the SM to itself (its passes and barriers leave the pipe idle: 16
+// warps use 75% of it, 8 warps 60%).
+struct F64Rate {
+  int ctas;
+  double t_pipe, t_alone;
+};
+F64Rate f64_rate(int n1, int n2, int n3, int T) {
+  const double N = (double)n1 * n2 * n3;
+  const int longest = std::max({n1, n2, n3});
+  const int threads = f64_cta_threads(n1, n2, n3, T);
+  const int regs = longest <= 12 ? 80 : longest <= 24 ? 128 : 256;
+  F64Rate r;
+  r.ctas = std::max(1, std::min({65536 / (regs * threads), (int)(kF64MaxSmem / (T * f64_grid_bytes(n1, n2, n3) + 1024)), 16}));
+  double warps = 0.0;
+  for (const int pencils : {n1 * n2, n1 * n3, n2 * n3}) warps += (double)((T * pencils + 31) / 32) * 32.0 / (3.0 * pencils);
+  r.t_pipe = warps * (10.0 * N * std::log2(N) + 16.0 * N) / 8e9;
+  r.t_alone = std::max((threads > 384 ? 1.32 : 1.6) * r.t_pipe, 4e-6);
+  r.t_pipe = std::max(r.t_pipe, r.t_alone / r.ctas);
+  return r;
+}
 constexpr double kWidePairSeconds = 7.1e-6;  // one partner of a tile of the two-exchange 16^3 kernel
 
 // Number of ranges the partners (k', j) of an owner tile are split into: the smallest estimated
 // time of list-scheduling `tiles` x ns ranges (partners / ns pairs of t_pair seconds, uneven where
-// ns does not divide, and 4 us an item for its start, owner and result) on `slots` resident CTAs,
-// plus the pass that sums the ranges' outputs (4 us and 3 TB/s over ns outputs).  A finer split
-// must gain 1%.  Beyond 48 waves the last one no longer matters.
+// ns does not divide, and t_item an item for its start, owner and result) on `slots` workers, plus
+// the pass that sums the ranges' outputs (4 us and 3 TB/s over ns outputs).  A worker is a
+// resident CTA, or an SM that several CTAs share; its last item then runs alone, t_tail a pair
+// longer.  A finer split must gain 1%.  Beyond 48 waves the last one no longer matters.
 struct SplitChoice {
   int ns = 1;
   double seconds = 0.0;
 };
 SplitChoice choose_split(long long tiles, long long partners, double t_pair, long long slots, size_t out_bytes,
-                         int ns_min) {
+                         int ns_min, double t_item = 4e-6, double t_tail = 0.0) {
   const int ns_cap = (int)std::min<long long>(32, partners);
   const long long most = 48 * slots;
   SplitChoice best;
@@ -477,11 +518,11 @@ SplitChoice choose_split(long long tiles, long long partners, double t_pair, lon
     if (best.seconds > 0.0 && (tiles * ns > most || (size_t)ns * out_bytes > ((size_t)4 << 30))) break;
     double t = 0.0;
     if (tiles * ns > most) {
-      t = (double)tiles * ((double)partners * t_pair + ns * 4e-6) / (double)slots;
+      t = (double)tiles * ((double)partners * t_pair + ns * t_item) / (double)slots;
     } else {
       std::map<double, long long> ends{{0.0, slots}};  // end time -> slots that end then
       for (int sp = 0; sp < ns; ++sp) {
-        const double cost = (double)((sp + 1) * partners / ns - sp * partners / ns) * t_pair + 4e-6;
+        const double cost = (double)((sp + 1) * partners / ns - sp * partners / ns) * t_pair + t_item;
         for (long long left = tiles; left > 0;) {  // the items of a range cost the same
           const auto first = ends.begin();
           const double end = first->first + cost;
@@ -493,6 +534,7 @@ SplitChoice choose_split(long long tiles, long long partners, double t_pair, lon
         }
       }
     }
+    t += t_tail * (double)((partners + ns - 1) / ns);
     if (ns > 1) t += 4e-6 + (double)ns * (double)out_bytes / 3e12;
     if (best.seconds == 0.0 || t < 0.99 * best.seconds) {
       best.seconds = t;
@@ -638,6 +680,7 @@ int hse_plan_destroy(hse_plan plan) {
   cudaFree(plan->partial);
   cudaFree(plan->status);
   cudaFree(plan->work);
+  cudaFree(plan->split64);
   cudaFree(plan->vx64);
   cudaFree(plan->split_buf);
   cudaFree(plan->comp_buf);
@@ -797,9 +840,54 @@ int hse_plan_create(hse_plan* out, const hse_problem* p) {
     }
     HSE_TRY(plan_malloc(plan, &plan->comp_buf, comp * sizeof(float2)));
   }
+  size_t e64_items = 0;
+  if (plan->p.dtype == HSE_C128 && f64_grid_bytes(n1, n2, n3) <= kF64MaxSmem) {
+    int sms = 0;
+    HSE_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, plan->device));
+    plan->sms = sms;
+    const int owners[3] = {p->n_tgt, p->n_occ, p->n_occ};
+    const int k_own[3] = {nk, nk, nkq};
+    const long long partners[3] = {(long long)nkq * p->n_occ,
+                                   plan->sampled ? (long long)nkq * p->n_occ : (long long)nk * p->n_occ / 2 + 1,
+                                   (long long)nk * p->n_tgt};
+    size_t buf = 0;
+    for (int o = 0; o < 3; ++o) {
+      const size_t out_bytes = o == ROLE_ENERGY ? 0 : (size_t)k_own[o] * owners[o] * N * sizeof(double2);
+      SplitChoice best;
+      for (const int T : {1, 2, 4, 8, 16}) {
+        if (T > 1 && (T * f64_grid_bytes(n1, n2, n3) > kF64MaxSmem || (T - 1) * std::max({n1 * n2, n1 * n3, n2 * n3}) >= 256))
+          break;
+        const F64Rate r = f64_rate(n1, n2, n3, T);
+        const long long tiles = o == ROLE_ENERGY ? ((long long)nk * p->n_occ + T - 1) / T
+                                                 : (long long)k_own[o] * ((owners[o] + T - 1) / T);
+        const double pass = o == ROLE_ENERGY ? 0.45 : o == ROLE_OCC ? 2.0 : 1.0;
+        const double t_pair = r.ctas > 1 ? r.t_pipe : r.t_alone;
+        const SplitChoice c = choose_split(tiles, partners[o], pass * t_pair, sms, out_bytes, 1, 4e-6 / r.ctas,
+                                           pass * (r.t_alone - t_pair));
+        if (T == 1 || c.seconds < 0.99 * best.seconds) {
+          best = c;
+          plan->f64_T[o] = T;
+        }
+      }
+      // the staged form: nine launches a target k-point, 0.93 TFLOP/s once they are full
+      const double pairs = (double)nk * owners[o] * nkq * p->n_occ * (o == ROLE_OCC ? 2.0 * p->n_tgt / p->n_occ : 1.0);
+      const double Nd = (double)N;
+      const double staged = nk * 9 * 6e-6 + pairs * (10.0 * Nd * std::log2(Nd) + 16.0 * Nd) / 0.93e12;
+      plan->fused64[o] = best.seconds < staged;
+      if (const char* env = std::getenv("HSE_FP64_FUSED")) plan->fused64[o] = std::atoi(env) != 0;
+      plan->f64_ns[o] = best.ns;
+      if (log_on())
+        std::fprintf(stderr, "hse: FP64 role %d: fused with %d orbitals a CTA and %d ranges %.0f us, staged %.0f us (estimates)\n",
+                     o, plan->f64_T[o], best.ns, best.seconds * 1e6, staged * 1e6);
+      if (plan->fused64[o] && best.ns > 1) buf = std::max(buf, best.ns * out_bytes);
+    }
+    if (buf) HSE_TRY(plan_malloc(plan, &plan->split64, buf));
+    if (plan->fused64[ROLE_ENERGY])
+      e64_items = (size_t)plan->f64_ns[ROLE_ENERGY] * (((size_t)nk * p->n_occ + plan->f64_T[ROLE_ENERGY] - 1) / plan->f64_T[ROLE_ENERGY]);
+  }
   {
-    const size_t np = std::max((size_t)plan->nsplit[ROLE_TGT] * nk * p->n_tgt,
-                               (size_t)plan->nsplit[ROLE_ENERGY] * nk * p->n_occ);
+    const size_t np = std::max({(size_t)plan->nsplit[ROLE_TGT] * nk * p->n_tgt,
+                                (size_t)plan->nsplit[ROLE_ENERGY] * nk * p->n_occ, e64_items});
     HSE_TRY(plan_malloc(plan, &plan->partial, std::max(np, (size_t)nk * nown) * sizeof(double)));
   }
   if (plan->sampled) {
@@ -828,7 +916,8 @@ int hse_plan_create(hse_plan* out, const hse_problem* p) {
     nkp = std::min<size_t>(nkp, (size_t)nkq);
     // at least two occupied x target batches: the VJP w.r.t. u_occ runs two at a time
     plan->work_pairs = std::max(nkp * per_kp, 2 * (size_t)p->n_occ * p->n_tgt);
-    HSE_TRY(plan_malloc(plan, &plan->work, plan->work_pairs * N * sizeof(double2)));
+    if (!plan->fused64[ROLE_TGT] || !plan->fused64[ROLE_ENERGY] || !plan->fused64[ROLE_OCC])
+      HSE_TRY(plan_malloc(plan, &plan->work, plan->work_pairs * N * sizeof(double2)));
     HSE_TRY(plan_malloc(plan, &plan->vx64, (size_t)nk * nown * N * sizeof(double2)));
   }
   TableArgs t{};
@@ -857,7 +946,7 @@ int hse_plan_create(hse_plan* out, const hse_problem* p) {
                  "k' splits target %d energy %d occupied %d; apply kernel %s; pencil-blocked copies %s\n",
                  n1, n2, n3, c64 ? "complex64" : "complex128", nk, nkq, p->n_occ, p->n_tgt, plan->nq,
                  plan->nsplit[ROLE_TGT], plan->nsplit[ROLE_ENERGY], plan->nsplit[ROLE_OCC],
-                 !c64 ? "staged FP64" : (pairconv_c64_pencil_load(n1, MODE_APPLY, plan->blocks_per_sm)
+                 !c64 ? (plan->fused64[ROLE_TGT] ? "fused FP64" : "staged FP64") : (pairconv_c64_pencil_load(n1, MODE_APPLY, plan->blocks_per_sm)
                                              ? (plan->tc ? "pencil-load, tensor-core Y/X" : "pencil-load")
                                              : plan->wide ? "two-exchange" : "staged-partner"),
                  plan->blocked ? "on" : "off");
@@ -1054,12 +1143,59 @@ int reduce(hse_plan plan, int n, double factor, double* out, cudaStream_t st, co
   return cuda_fail(cudaGetLastError());
 }
 
-// Staged FP64 V_x: out[k][i] for every target; table = v64 or dv64.  u_occ / occ are the
-// occupied rows of the Fock sum ([nkq][n_occ]).
-int staged_apply(hse_plan plan, const double2* u_occ, const double* occ, const double2* u_tgt, int n_tgt,
-                 const double* table, double2* out, cudaStream_t st) {
+// Arguments of the fused FP64 kernel for one owner role; owners and partners as in the complex64
+// launches.
+F64Args f64_args(hse_plan plan, FusedMode mode, int role) {
+  const hse_problem& p = plan->p;
+  F64Args a{};
+  a.mode = mode;
+  a.n1 = p.grid[0];
+  a.n2 = p.grid[1];
+  a.n3 = p.grid[2];
+  a.N = plan->N;
+  a.qidx = plan->qidx;
+  a.vtab = plan->v64;
+  a.n_occ = p.n_occ;
+  a.nk_own = role == ROLE_OCC ? plan->nkq : p.nk;
+  a.nk_part = role == ROLE_OCC ? p.nk : plan->nkq;
+  a.n_own = role == ROLE_TGT ? p.n_tgt : p.n_occ;
+  a.n_part = role == ROLE_OCC ? p.n_tgt : p.n_occ;
+  a.T = plan->f64_T[role];
+  a.nsplit = plan->f64_ns[role];
+  a.stagger = plan->sms;
+  a.ntiles = (a.n_own + a.T - 1) / a.T;
+  a.scale = -p.alpha / ((double)plan->nkq * plan->N);
+  return a;
+}
+
+// Launch of an APPLY or OCC pass into `out`, with the sum over the splits.
+int run_fused64(hse_plan plan, F64Args a, double2* out, cudaStream_t st) {
+  a.out = a.nsplit > 1 ? plan->split64 : out;
+  cudaError_t e = launch_fused_f64(a, st);
+  if (e == cudaSuccess && a.nsplit > 1) {
+    const size_t count = (size_t)a.nk_own * a.n_own * a.N;
+    reduce_splits_f64<<<(unsigned)std::min<size_t>((count + 255) / 256, 152 * 16), 256, 0, st>>>(out, plan->split64,
+                                                                                               a.nsplit, count);
+    count_launch();
+    e = cudaGetLastError();
+  }
+  return cuda_fail(e);
+}
+
+// FP64 V_x: out[k][i] for every target; table = v64 or dv64.  u_occ / occ are the occupied rows of
+// the Fock sum ([nkq][n_occ]).  fused: by the fused kernel (the plan's choice for these owners).
+int apply_f64(hse_plan plan, const double2* u_occ, const double* occ, const double2* u_tgt, int n_tgt,
+                 const double* table, double2* out, bool fused, cudaStream_t st) {
   const hse_problem& p = plan->p;
   const int N = plan->N;
+  if (fused) {
+    F64Args a = f64_args(plan, F64_APPLY, ROLE_TGT);
+    a.own = u_tgt;
+    a.part = u_occ;
+    a.occ = occ;
+    a.vtab = table;
+    return run_fused64(plan, a, out, st);
+  }
   const int nk = p.nk, nkq = plan->nkq;
   const size_t per_kp = (size_t)n_tgt * p.n_occ;
   if (per_kp > plan->work_pairs) return HSE_ERR_INVALID_ARG;  // cannot happen: sized for max(n_occ, n_tgt)
@@ -1228,11 +1364,11 @@ int staged_vjp(hse_plan plan, const double2* u_occ, const double* occ, const dou
   const int N = plan->N;
   int rc = HSE_OK;
   if (g_tgt) {
-    rc = staged_apply(plan, u_occ, occ, ybar, p.n_tgt, plan->v64, g_tgt, st);
+    rc = apply_f64(plan, u_occ, occ, ybar, p.n_tgt, plan->v64, g_tgt, plan->fused64[ROLE_TGT], st);
     if (rc) return rc;
   }
   if (g_om) {
-    rc = staged_apply(plan, u_occ, occ, u_tgt, p.n_tgt, plan->dv64, plan->vx64, st);
+    rc = apply_f64(plan, u_occ, occ, u_tgt, p.n_tgt, plan->dv64, plan->vx64, plan->fused64[ROLE_TGT], st);
     if (rc) return rc;
     dot_per_owner_f64<<<p.nk * p.n_tgt, 256, 0, st>>>(ybar, plan->vx64, N, nullptr, plan->partial);
     count_launch();
@@ -1240,6 +1376,14 @@ int staged_vjp(hse_plan plan, const double2* u_occ, const double* occ, const dou
     if (rc) return rc;
     rc = reduce(plan, p.nk * p.n_tgt, 1.0, g_om, st);
     if (rc) return rc;
+  }
+  if (g_occ && plan->fused64[ROLE_OCC]) {
+    F64Args a = f64_args(plan, F64_OCC, ROLE_OCC);
+    a.own = u_occ;
+    a.part = u_tgt;
+    a.part2 = ybar;
+    a.occ = occ;
+    return run_fused64(plan, a, g_occ, st);
   }
   if (g_occ) {
     // the work buffer holds two pair batches of work_pairs / 2 each
@@ -1317,8 +1461,8 @@ int hse_fock_apply(hse_plan plan, const void* u_occ, const double* occ, const vo
     a.n_part = p.n_occ;
     return run_pairconv(plan, MODE_APPLY, a, p.n_tgt, st);
   }
-  return staged_apply(plan, (const double2*)u_rows, occ_rows, (const double2*)u_tgt, p.n_tgt, plan->v64,
-                      (double2*)vx_out, st);
+  return apply_f64(plan, (const double2*)u_rows, occ_rows, (const double2*)u_tgt, p.n_tgt, plan->v64,
+                      (double2*)vx_out, plan->fused64[ROLE_TGT], st);
 }
 
 int hse_exchange_energy(hse_plan plan, const void* u_occ, const double* occ, double* e_x, hse_stream_t stream) {
@@ -1343,9 +1487,21 @@ int hse_exchange_energy(hse_plan plan, const void* u_occ, const double* occ, dou
     a.occ_own = occ;
     a.n_part = p.n_occ;
     rc = run_pairconv(plan, MODE_ENERGY, a, p.n_occ, st);
+  } else if (plan->fused64[ROLE_ENERGY]) {
+    F64Args a = f64_args(plan, F64_ENERGY, ROLE_ENERGY);
+    a.own = (const double2*)u_occ;
+    a.part = (const double2*)u_rows;
+    a.occ = occ_rows;
+    a.occ_own = occ;
+    a.sym = plan->sampled ? 0 : 1;
+    a.partial = plan->partial;
+    a.ntiles = (nown + a.T - 1) / a.T;
+    rc = cuda_fail(launch_fused_f64(a, st));
+    if (rc) return rc;
+    return reduce(plan, a.nsplit * a.ntiles, factor, e_x, st);
   } else {
-    rc = staged_apply(plan, (const double2*)u_rows, occ_rows, (const double2*)u_occ, p.n_occ, plan->v64, plan->vx64,
-                      st);
+    rc = apply_f64(plan, (const double2*)u_rows, occ_rows, (const double2*)u_occ, p.n_occ, plan->v64, plan->vx64,
+                      false, st);
     if (rc) return rc;
     dot_per_owner_f64<<<nown, 256, 0, st>>>((const double2*)u_occ, plan->vx64, plan->N, occ, plan->partial);
     count_launch();
