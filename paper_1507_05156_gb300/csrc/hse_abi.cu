@@ -341,6 +341,8 @@ struct hse_plan_s {
   double2* hart_work = nullptr;   // Hartree potential: [N] FP64 transform
   double2* ortho_work = nullptr;  // orthonormalisation of complex64 orbitals: FP64 copy
   size_t ortho_elems = 0;
+  void* ortho_scratch = nullptr;  // overlap matrices, factors and flags of the orthonormalisation
+  size_t ortho_scratch_size = 0;
   // batched plans (hse_plan_create_batched)
   bool batched = false;
   std::vector<hse_plan> cells;          // one sub-plan (kernel tables) per cell
@@ -696,6 +698,7 @@ int hse_plan_destroy(hse_plan plan) {
   cudaFree(plan->cur_work);
   cudaFree(plan->cur_partial);
   cudaFree(plan->hart_work);
+  cudaFree(plan->ortho_scratch);
   cudaFree(plan->ortho_work);
   cudaSetDevice(prev);
   delete plan;
@@ -1707,8 +1710,17 @@ int hse_orthonormalize(hse_plan plan, void* u, int nbands, hse_stream_t stream) 
     if (e != cudaSuccess) return cuda_fail(e);
     plan->ortho_elems = count;
   }
+  const size_t scratch = ortho_scratch_bytes(p.nk, nbands);
+  if (scratch > plan->ortho_scratch_size) {
+    cudaFree(plan->ortho_scratch);
+    plan->ortho_scratch = nullptr;
+    plan->ortho_scratch_size = 0;
+    const cudaError_t e = plan_malloc(plan, &plan->ortho_scratch, scratch);
+    if (e != cudaSuccess) return cuda_fail(e);
+    plan->ortho_scratch_size = scratch;
+  }
   return cuda_fail(launch_orthonormalize(p.dtype == HSE_C128, u, p.nk, nbands, plan->N, plan->dV, plan->ortho_work,
-                                         plan->status, S(stream)));
+                                         plan->ortho_scratch, plan->status, S(stream)));
 }
 
 int hse_hartree_potential(hse_plan plan, const void* psi, const double* occ, double* vh, hse_stream_t stream) {

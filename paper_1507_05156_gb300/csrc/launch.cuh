@@ -42,10 +42,12 @@ constexpr int kStatusSingular = -8;  // HSE_ERR_SINGULAR
 // S device [nk][nb][nb] double2: S[k][a][b] = dV sum_r conj(u_{a,k}) u_{b,k}
 cudaError_t launch_overlap(bool c128, const void* u, int nk, int nb, size_t N, double dV, double2* S,
                            cudaStream_t stream);
-// u [nk][nb][N] in place (two modified Gram-Schmidt passes); work: [nk][nb][N] double2
-// scratch for complex64 orbitals (unused for complex128); status: the plan's status word.
-cudaError_t launch_orthonormalize(bool c128, void* u, int nk, int nb, size_t N, double dV, double2* work, int* status,
-                                  cudaStream_t stream);
+// u [nk][nb][N] in place (two modified Gram-Schmidt passes, or their equal); work: [nk][nb][N]
+// double2 scratch for complex64 orbitals (unused for complex128); scratch: ortho_scratch_bytes;
+// status: the plan's status word.
+size_t ortho_scratch_bytes(int nk, int nb);
+cudaError_t launch_orthonormalize(bool c128, void* u, int nk, int nb, size_t N, double dV, double2* work, void* scratch,
+                                  int* status, cudaStream_t stream);
 
 // Fused complex64 pair-convolution launch for a cubic grid of side n (one TU per size
 // group keeps the build parallel).  Returns a cudaError_t.
