@@ -476,10 +476,10 @@ double pair_seconds(int n) {
   const double N = (double)n * n * n;
   return (10.0 * N * std::log2(N) + 16.0 * N) / 0.27e12;
 }
-// The fused FP64 kernel with T orbitals a CTA: CTAs an SM holds, seconds of its FP64 pipe a partner
-// takes (about 8 GFLOP/s of the same count, a partial warp costing a whole one), and seconds a
-// partner takes in a CTA that has the SM to itself (its passes and barriers leave the pipe idle: 16
-// warps use 75% of it, 8 warps 60%).
+// The fused FP64 kernel with T orbitals a CTA: CTAs an SM holds, seconds of an SM a partner takes
+// when they are all busy (6.5 GFLOP/s of the same count; a partial warp costs a whole one, and with
+// one or two CTAs so does a scheduler without a warp in a pass's last round), and seconds a partner
+// takes in a CTA whose SM holds no other.
 struct F64Rate {
   int ctas;
   double t_pipe, t_alone;
@@ -492,9 +492,10 @@ F64Rate f64_rate(int n1, int n2, int n3, int T) {
   F64Rate r;
   r.ctas = std::max(1, std::min({65536 / (regs * threads), (int)(kF64MaxSmem / (T * f64_grid_bytes(n1, n2, n3) + 1024)), 16}));
   double warps = 0.0;
-  for (const int pencils : {n1 * n2, n1 * n3, n2 * n3}) warps += (double)((T * pencils + 31) / 32) * 32.0 / (3.0 * pencils);
-  r.t_pipe = warps * (10.0 * N * std::log2(N) + 16.0 * N) / 8e9;
-  r.t_alone = std::max((threads > 384 ? 1.32 : 1.6) * r.t_pipe, 4e-6);
+  const int step = r.ctas <= 2 ? 128 : 32;
+  for (const int pencils : {n1 * n2, n1 * n3, n2 * n3}) warps += (double)((T * pencils + step - 1) / step * step) / (3.0 * pencils);
+  r.t_pipe = warps * (10.0 * N * std::log2(N) + 16.0 * N) / 6.5e9;
+  r.t_alone = std::max((r.ctas > 1 ? 1.25 : 1.0) * r.t_pipe, 4e-6);
   r.t_pipe = std::max(r.t_pipe, r.t_alone / r.ctas);
   return r;
 }
@@ -865,18 +866,18 @@ int hse_plan_create(hse_plan* out, const hse_problem* p) {
                                                  : (long long)k_own[o] * ((owners[o] + T - 1) / T);
         const double pass = o == ROLE_ENERGY ? 0.45 : o == ROLE_OCC ? 2.0 : 1.0;
         const double t_pair = r.ctas > 1 ? r.t_pipe : r.t_alone;
-        const SplitChoice c = choose_split(tiles, partners[o], pass * t_pair, sms, out_bytes, 1, 4e-6 / r.ctas,
+        const SplitChoice c = choose_split(tiles, partners[o], pass * t_pair, sms, out_bytes, 1, 1.5e-6 / r.ctas,
                                            pass * (r.t_alone - t_pair));
         if (T == 1 || c.seconds < 0.99 * best.seconds) {
           best = c;
           plan->f64_T[o] = T;
         }
       }
-      // the staged form: nine launches a target k-point, 0.93 TFLOP/s once they are full
+      // the staged form: nine launches a target k-point, 0.84 TFLOP/s once they are full (0.93 at 24^3)
       const double pairs = (double)nk * owners[o] * nkq * p->n_occ * (o == ROLE_OCC ? 2.0 * p->n_tgt / p->n_occ : 1.0);
       const double Nd = (double)N;
-      const double staged = nk * 9 * 6e-6 + pairs * (10.0 * Nd * std::log2(Nd) + 16.0 * Nd) / 0.93e12;
-      plan->fused64[o] = best.seconds < staged;
+      const double staged = nk * 9 * 6e-6 + pairs * (10.0 * Nd * std::log2(Nd) + 16.0 * Nd) / (N > 8000 ? 0.93e12 : 0.84e12);
+      plan->fused64[o] = best.seconds < 0.97 * staged;
       if (const char* env = std::getenv("HSE_FP64_FUSED")) plan->fused64[o] = std::atoi(env) != 0;
       plan->f64_ns[o] = best.ns;
       if (log_on())
