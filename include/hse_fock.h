@@ -248,10 +248,11 @@ int hse_hartree_potential(hse_plan plan, const void *psi, const double *occ, dou
  * absorbed into A):
  *   J = -(1/Omega) int_Omega sum_i w_i Re[psi_i* (-i grad + A) psi_i]
  *     = -sum_{k,i} (g_s f_{i,k} / N_k) sum_G |c_{i,k}(G)|^2 (G + k + A),
- * c = (1/N) sum_r u(r) e^{-iG.r}, computed with FP64 transforms and reduced in FP64.
+ * c = (1/N) sum_r u(r) e^{-iG.r}, with FP64 transforms and sums (each axis of G by 1-D transforms along it,
+ * Parseval over the other two).
  *   psi  device [nk][n_occ][N] (the plan's dtype), occ device [nk][n_occ]
  *   A    HOST [3];  J  device double[3], overwritten
- * g_s is the plan's spin_degeneracy.  The first call allocates an FP64 copy of the orbitals
+ * g_s is the plan's spin_degeneracy.  The first call allocates four doubles an orbital
  * in the plan; later calls are asynchronous on `stream`.  Not for batched plans. */
 int hse_current(hse_plan plan, const void *psi, const double *occ, const double *A, double *J,
                 hse_stream_t stream);

@@ -336,8 +336,7 @@ struct hse_plan_s {
   void* g_sub = nullptr;        // device [nkq][n_occ][N] VJP w.r.t. the sampled orbitals
   // time propagation (allocated on first use)
   void* tay[3] = {nullptr, nullptr, nullptr};  // Taylor step: term, T term, V_x term [nk][n_occ][N]
-  double2* cur_work = nullptr;  // current: FP64 transforms [nk][n_occ][N]
-  double* cur_partial = nullptr;  // current: [nk][n_occ][3]
+  double* cur_partial = nullptr;  // current: moments [nk][n_occ][4]
   double2* hart_work = nullptr;   // Hartree potential: [N] FP64 transform
   double2* ortho_work = nullptr;  // orthonormalisation of complex64 orbitals: FP64 copy
   size_t ortho_elems = 0;
@@ -696,7 +695,6 @@ int hse_plan_destroy(hse_plan plan) {
   cudaFree(plan->occ_sub);
   cudaFree(plan->g_sub);
   for (void* b : plan->tay) cudaFree(b);
-  cudaFree(plan->cur_work);
   cudaFree(plan->cur_partial);
   cudaFree(plan->hart_work);
   cudaFree(plan->ortho_scratch);
@@ -1644,16 +1642,15 @@ int hse_taylor_step(hse_plan plan, const void* psi, const double* occ, const dou
       if (e != cudaSuccess) return cuda_fail(e);
     }
   cudaStream_t st = S(stream);
-  cudaError_t e = cudaMemcpyAsync(psi_out, psi, bytes, cudaMemcpyDeviceToDevice, st);
-  if (e != cudaSuccess) return cuda_fail(e);
   const void* term = psi;
   for (int n = 1; n <= 4; ++n) {
     int rc = hse_kinetic_apply(plan, term, p.n_occ, A, plan->tay[1], stream);
     if (rc) return rc;
     rc = hse_fock_apply(plan, psi, occ, term, plan->tay[2], stream);
     if (rc) return rc;
-    e = launch_taylor_accumulate(p.dtype == HSE_C128, plan->tay[1], plan->tay[2], term, vloc, (size_t)plan->N,
-                                 plan->tay[0], psi_out, count, dt / n, st);
+    const cudaError_t e = launch_taylor_accumulate(p.dtype == HSE_C128, plan->tay[1], plan->tay[2], term, vloc,
+                                                   (size_t)plan->N, plan->tay[0], n == 1 ? psi : psi_out, psi_out, count,
+                                                   dt / n, st);
     if (e != cudaSuccess) return cuda_fail(e);
     term = plan->tay[0];
   }
@@ -1668,9 +1665,8 @@ int hse_current(hse_plan plan, const void* psi, const double* occ, const double*
   if (!aligned16(psi)) return HSE_ERR_INVALID_ARG;
   const hse_problem& p = plan->p;
   const size_t norb = (size_t)p.nk * p.n_occ;
-  if (!plan->cur_work) {
-    cudaError_t e = plan_malloc(plan, &plan->cur_work, norb * plan->N * sizeof(double2));
-    if (e == cudaSuccess) e = plan_malloc(plan, &plan->cur_partial, norb * 3 * sizeof(double));
+  if (!plan->cur_partial) {
+    const cudaError_t e = plan_malloc(plan, &plan->cur_partial, norb * 4 * sizeof(double));
     if (e != cudaSuccess) return cuda_fail(e);
   }
   CurArgs a{};
@@ -1682,8 +1678,8 @@ int hse_current(hse_plan plan, const void* psi, const double* occ, const double*
   std::memcpy(a.b, plan->b, sizeof(a.b));
   for (int c = 0; c < 3; ++c) a.A[c] = A[c];
   a.kpts = plan->dkpts;
-  return cuda_fail(launch_current(p.dtype == HSE_C128, psi, occ, a, plan->cur_work, plan->cur_partial,
-                                  p.spin_degeneracy, J, S(stream)));
+  return cuda_fail(launch_current(p.dtype == HSE_C128, psi, occ, a, plan->cur_partial, p.spin_degeneracy, J,
+                                  S(stream)));
 }
 
 int hse_overlap(hse_plan plan, const void* u, int nbands, double* s_out, hse_stream_t stream) {

@@ -28,14 +28,15 @@ struct CurArgs {
   const double* kpts;   // device [nk][3]
 };
 cudaError_t launch_taylor_accumulate(bool c128, const void* kin, const void* vx, const void* prev, const double* vloc,
-                                     size_t N, void* term, void* out, size_t count, double s, cudaStream_t stream);
+                                     size_t N, void* term, const void* base, void* out, size_t count, double s,
+                                     cudaStream_t stream);
 // v_H (device double [N]) of the orbitals' density; work: [N] double2 scratch.
 cudaError_t launch_hartree(bool c128, const void* psi, const double* occ, const CurArgs& a, double spin_degeneracy,
                            double2* work, double* vh, cudaStream_t stream);
 // J (device double[3]) from the orbitals psi [nk][nbands][N] and occupations [nk][nbands];
-// work: [nk][nbands][N] double2 scratch, partial: [nk][nbands][3] double scratch.
-cudaError_t launch_current(bool c128, const void* psi, const double* occ, const CurArgs& a, double2* work,
-                           double* partial, double spin_degeneracy, double* J, cudaStream_t stream);
+// partial: [nk][nbands][4] double scratch.
+cudaError_t launch_current(bool c128, const void* psi, const double* occ, const CurArgs& a, double* partial,
+                           double spin_degeneracy, double* J, cudaStream_t stream);
 
 // Overlap matrices and Gram-Schmidt orthonormalisation in FP64 (ortho.cu).
 constexpr int kStatusSingular = -8;  // HSE_ERR_SINGULAR
