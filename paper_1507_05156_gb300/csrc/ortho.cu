@@ -110,9 +110,10 @@ __device__ __forceinline__ void gram_point(double2 (&acc)[4][4], const double2 (
 // CTAs over the points, k, groups of kGramTiles tiles); a warp takes tile warp % kGramTiles' share
 // (tiles of this group) and every R-th run of 32 points.
 // The FP64 pipe bounds it: 64 multiply-adds a tile and point (32 on the diagonal) against eight
-// shared-memory reads; the values are widened once per CTA, when staged.
+// shared-memory reads; the values are widened once per CTA, when staged.  Two CTAs an SM (96
+// registers, a few spills) fill each other's barriers: 64 k x 16 bands at 20^3 989 -> 650 us.
 template <typename C>
-__global__ void gram_kernel(const C* __restrict__ u, int nb, size_t N, double dV, double2* __restrict__ S, int tiles_here,
+__global__ void __launch_bounds__(32 * kGramTiles, 2) gram_kernel(const C* __restrict__ u, int nb, size_t N, double dV, double2* __restrict__ S, int tiles_here,
                             int R, const int* __restrict__ skip) {
   extern __shared__ __align__(16) double2 stg[];  // [nbp][32 R]
   __shared__ double red[kGramTiles][33];
@@ -120,7 +121,10 @@ __global__ void gram_kernel(const C* __restrict__ u, int nb, size_t N, double dV
   const int k = blockIdx.y, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (skip && skip[k]) return;  // uniform over the cluster
   const int nt = (nb + 3) / 4, ntiles = nt * (nt + 1) / 2, P = 32 * R;
-  const int tl = warp % tiles_here, rep = warp / tiles_here;
+  // 16 bands: diagonal tiles (0, 4, 7, 9; half the work) go to the schedulers that hold three warps
+  constexpr unsigned long long kOrder16 = 0x9786405321ull;
+  const int wt = warp % tiles_here, rep = warp / tiles_here;
+  const int tl = ntiles == 10 ? (int)((kOrder16 >> (4 * wt)) & 15) : wt;
   const bool on = (int)blockIdx.z * kGramTiles + tl < ntiles;
   int ti = 0, left = on ? blockIdx.z * kGramTiles + tl : 0;
   while (left >= nt - ti) left -= nt - ti++;  // tiles row by row, tj >= ti
@@ -194,7 +198,7 @@ __global__ void gram_kernel(const C* __restrict__ u, int nb, size_t N, double dV
     double s = 0.0;
     for (int c = 0; c < (int)cl.num_blocks(); ++c) {
       const double* remote = cl.map_shared_rank(&red[0][0], c);
-      for (int p = 0; p < R; ++p) s += remote[(p * tiles_here + tl) * 33 + lane];
+      for (int p = 0; p < R; ++p) s += remote[(p * tiles_here + wt) * 33 + lane];
     }
     s *= dV;
     const int a = 4 * ti + (lane >> 3), b = 4 * tj + ((lane >> 1) & 3), part = lane & 1;
@@ -233,7 +237,7 @@ __global__ void gram_factor(const double2* __restrict__ S, int nb, double2* __re
   for (int i = tid; i < nb * nb; i += blockDim.x) {
     const int d = i / nb, a = i - d * nb;
     lm[i] = d >= a ? Sk[(size_t)a * nb + d] : make_double2(0.0, 0.0);
-    tm[i] = make_double2(0.0, 0.0);
+    tm[i] = make_double2(d == a ? 1.0 : 0.0, 0.0);
   }
   __syncthreads();
   for (int a = 0; a < nb; ++a) {
@@ -243,35 +247,33 @@ __global__ void gram_factor(const double2* __restrict__ S, int nb, double2* __re
     __syncthreads();
     for (int d = a + tid; d < nb; d += blockDim.x)
       lm[d * nb + a] = d == a ? make_double2(p * inv, 0.0) : make_double2(lm[d * nb + a].x * inv, lm[d * nb + a].y * inv);
+    for (int b = tid; b <= a; b += blockDim.x) {  // row a of T is final
+      tm[a * nb + b].x *= inv;
+      tm[a * nb + b].y *= inv;
+    }
     __syncthreads();
-    // trailing update: S_ef -= conj(L_ea) L_fa at lm[f][e], f >= e > a
+    // rows f > a: S_ef -= conj(L_ea) L_fa at lm[f][e] for f >= e > a, and T_fe -= L_fa T_ae for e <= a
     const int m = nb - a - 1;
-    for (int i = tid; i < m * m; i += blockDim.x) {
-      const int f = a + 1 + i / m, e = a + 1 + i % m;
+    for (int i = tid; i < m * nb; i += blockDim.x) {
+      const int f = a + 1 + i / nb, e = i % nb;
       if (f < e) continue;
-      const double2 x = lm[e * nb + a], y = lm[f * nb + a];
-      lm[f * nb + e].x -= x.x * y.x + x.y * y.y;
-      lm[f * nb + e].y -= x.x * y.y - x.y * y.x;
+      const double2 y = lm[f * nb + a];
+      if (e > a) {
+        const double2 x = lm[e * nb + a];
+        lm[f * nb + e].x -= x.x * y.x + x.y * y.y;
+        lm[f * nb + e].y -= x.x * y.y - x.y * y.x;
+      } else {
+        const double2 x = tm[a * nb + e];
+        tm[f * nb + e].x -= x.x * y.x - x.y * y.y;
+        tm[f * nb + e].y -= x.x * y.y + x.y * y.x;
+      }
     }
     __syncthreads();
   }
-  // columns of L^-1, one thread each: T_ab = -(1 / L_aa) sum_{b <= c < a} L_ac T_cb
   double mine = 0.0;
-  for (int b = tid; b < nb; b += blockDim.x) {
-    const double sb = Sk[(size_t)b * nb + b].x;
-    for (int a = b; a < nb; ++a) {
-      double2 s = make_double2(a == b ? 1.0 : 0.0, 0.0);
-      for (int c = b; c < a; ++c) {
-        const double2 l = lm[a * nb + c], t = tm[c * nb + b];
-        s.x -= l.x * t.x - l.y * t.y;
-        s.y -= l.x * t.y + l.y * t.x;
-      }
-      const double inv = 1.0 / lm[a * nb + a].x;
-      s.x *= inv;
-      s.y *= inv;
-      tm[a * nb + b] = s;
-      mine += (s.x * s.x + s.y * s.y) * sb;
-    }
+  for (int i = tid; i < nb * nb; i += blockDim.x) {
+    const int b = i % nb;
+    mine += (tm[i].x * tm[i].x + tm[i].y * tm[i].y) * Sk[(size_t)b * nb + b].x;
   }
   if (mine != 0.0) atomicAdd(&cond, mine);  // only compared with a bound: the order does not matter
   __syncthreads();
