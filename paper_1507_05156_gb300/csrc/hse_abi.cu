@@ -306,7 +306,8 @@ struct hse_plan_s {
   bool blocked = true;       // pencil-load launches read pencil-blocked copies (HSE_PENCIL_BLOCKS=0: no)
   int blocks_per_sm = 0;     // fused-kernel variant: 0 default, -1/-2 staged-partner layouts, 1/2/3/5 pencil loads,
                              // kTcVariant the tensor-core form (HSE_C64_TC)
-  bool wide = false;         // the apply runs the two-exchange 16^3 kernel (kWideVariant)
+  bool wide = false;         // the apply runs the two-exchange 16^3 kernel (kWideVariant),
+  bool wide_occ = false;     // and so does the VJP's u_occ pass
   bool tc = false;           // created as HSE_C64_TC (p.dtype then reads HSE_C64)
   int inject = 0;            // test hook (HSE_INJECT_SKIP_FILL=1 at plan creation)
   long long alloc_count = 0;   // device allocations made by this plan so far (plan_malloc)
@@ -498,7 +499,9 @@ F64Rate f64_rate(int n1, int n2, int n3, int T) {
   r.t_pipe = std::max(r.t_pipe, r.t_alone / r.ctas);
   return r;
 }
-constexpr double kWidePairSeconds = 7.1e-6;  // one partner of a tile of the two-exchange 16^3 kernel
+constexpr double kWidePairSeconds = 7.1e-6;  // one partner of a tile of the two-exchange 16^3 kernel,
+constexpr double kWideOccSeconds = 17e-6;  // of its u_occ pass (two chains; 14.7 without omega, 18 with),
+constexpr double kPencilOccSeconds16 = 9.4e-6;  // and of the pencil-load kernel's u_occ pass (a two-owner tile)
 
 // Number of ranges the partners (k', j) of an owner tile are split into: the smallest estimated
 // time of list-scheduling `tiles` x ns ranges (partners / ns pairs of t_pair seconds, uneven where
@@ -740,7 +743,7 @@ int hse_plan_create(hse_plan* out, const hse_problem* p) {
   if (const char* env = std::getenv("HSE_BLOCKS_PER_SM")) {
     const int v = std::atoi(env);
     plan->blocks_per_sm = (v < -2 || v > kOneVariant || v == kTcVariant) ? 0 : v;
-    plan->wide = v == kWideVariant && p->dtype == HSE_C64 && p->grid[0] == 16;  // also where it is slower
+    plan->wide = plan->wide_occ = v == kWideVariant && p->dtype == HSE_C64 && p->grid[0] == 16;  // also where it is slower
   }
   if (plan->tc) plan->blocks_per_sm = kTcVariant;
   const int n1 = p->grid[0], n2 = p->grid[1], n3 = p->grid[2];
@@ -825,6 +828,12 @@ int hse_plan_create(hse_plan* out, const hse_problem* p) {
         const SplitChoice wide = choose_split(tiles(kWideSlots), partners, kWidePairSeconds, sms, out_bytes, ns_min);
         plan->wide = plan->wide || wide.seconds < choice.seconds;
         if (plan->wide) choice = wide;
+      }
+      if (o == ROLE_OCC && n1 == 16 && plan->blocks_per_sm == 0) {
+        const SplitChoice wide = choose_split(tiles(kWideSlots), partners, kWideOccSeconds, sms, out_bytes, ns_min);
+        choice = choose_split(tiles(T), partners, kPencilOccSeconds16, slots, out_bytes, ns_min);
+        plan->wide_occ = plan->wide_occ || wide.seconds < choice.seconds;
+        if (plan->wide_occ) choice = wide;
       }
       int best = choice.ns;
       size_t need = (best > 1 && o != ROLE_ENERGY) ? (size_t)best * k_own[o] * owners[o] * N : 0;
@@ -1037,12 +1046,17 @@ int to_blocked(hse_plan plan, int mode, PairArgs& a, cudaStream_t st) {
   return cuda_fail(cudaGetLastError());
 }
 
+// Kernel variant of a pass: the plan's, or the two-exchange kernel where it chose that.
+int kernel_variant(hse_plan plan, int mode) {
+  return (mode == MODE_APPLY && plan->wide) || (mode == MODE_OCC && plan->wide_occ) ? kWideVariant : plan->blocks_per_sm;
+}
+
 int run_pairconv(hse_plan plan, int mode, PairArgs a, int n_own, cudaStream_t st) {
   const int n = plan->p.grid[0];
-  const int variant = mode == MODE_APPLY && plan->wide ? kWideVariant : plan->blocks_per_sm;
+  const int variant = kernel_variant(plan, mode);
   const int T = owner_slots(n, variant);
   a.n_own = n_own;
-  if (pairconv_c64_pencil_load(n, mode, plan->blocks_per_sm) && plan->blocked) {
+  if (variant != kWideVariant && pairconv_c64_pencil_load(n, mode, variant) && plan->blocked) {
     const int rc = to_blocked(plan, mode, a, st);
     if (rc) return rc;
   }
@@ -1062,7 +1076,7 @@ int run_pairconv(hse_plan plan, int mode, PairArgs a, int n_own, cudaStream_t st
     // the omega gradient fused into the u_occ pass: launches of at most kSpecCtas CTAs, each
     // CTA with its own spectrum scratch, and one FP64 partial per item
     const long long items = (long long)a.nsplit * a.nk_own * a.ntiles;
-    const size_t per_cta = (size_t)slots_for(n) * blocked_stride(n);
+    const size_t per_cta = (size_t)T * blocked_stride(n);
     const size_t spec_need = (size_t)std::min<long long>(items, kSpecCtas) * per_cta;
     if (spec_need > plan->spec_elems) {
       cudaFree(plan->spec_buf);
@@ -1586,7 +1600,7 @@ int hse_fock_apply_vjp(hse_plan plan, const void* u_occ, const double* occ, cons
     if (fuse_w) a.vtab2 = plan->dv32;
     rc = run_pairconv(plan, MODE_OCC, a, p.n_occ, st);
     if (rc == HSE_OK && fuse_w) {
-      const int T = slots_for(p.grid[0]);
+      const int T = owner_slots(p.grid[0], kernel_variant(plan, MODE_OCC));
       const int items = plan->nsplit[ROLE_OCC] * plan->nkq * ((p.n_occ + T - 1) / T);
       rc = reduce(plan, items, 1.0, grad_omega, st, plan->wpartial);
     }

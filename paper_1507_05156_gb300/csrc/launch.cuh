@@ -206,7 +206,7 @@ constexpr bool pencil_one_fits() {
 cudaError_t make_partner_tmap(CUtensorMap* map, const void* base, int n, long long rows, int sp, int box_rows,
                               bool swizzle = false);
 
-// Two-exchange kernel of the 16^3 apply (kWideVariant, pairconv_wide.cuh): four owners a CTA.  A
+// Two-exchange kernels of the 16^3 apply and u_occ pass (kWideVariant, pairconv_wide.cuh): four owners a CTA.  A
 // pair of its tile takes 7.1 us however few of the four slots are filled (two warps a scheduler
 // that mostly wait for themselves), a pair of the staged kernel's two-owner tile 4.1 us; so it is
 // for plans with enough tiles, which choose it by estimated time (hse_plan_create): 12^3
@@ -214,7 +214,7 @@ cudaError_t make_partner_tmap(CUtensorMap* map, const void* base, int n, long lo
 // 73 us against 55 us staged.
 constexpr int kWideVariant = 6;
 constexpr int kWideSlots = 4;
-cudaError_t launch_pairconv_wide16(const PairArgs& args, cudaStream_t stream);
+cudaError_t launch_pairconv_wide16(int mode, const PairArgs& args, cudaStream_t stream);  // MODE_APPLY, MODE_OCC
 // owner orbitals per work item of the kernel that (n, variant) runs
 constexpr int owner_slots(int n, int variant) { return variant == kWideVariant ? kWideSlots : slots_for(n); }
 
@@ -258,7 +258,7 @@ constexpr bool tma_fits() {
 // (pencil_ragged_fits; 24^3 99.6 -> 95.6 ms on the 4x4x4 k, 16-band cell against two pencils a
 // thread on 9 warps); 4 (kTcVariant) its tensor-core form where tc_fits, else the ragged
 // kernel; 5 (kOneVariant) the one-pencil pencil-load kernel where pencil_one_fits; 6
-// (kWideVariant) the two-exchange kernel (16^3 apply only; chosen by the plan).
+// (kWideVariant) the two-exchange kernels (16^3 apply and u_occ pass; chosen by the plan).
 // A variant that does not exist for the size falls back to the default.
 template <int n, int MODE>
 constexpr int staged_layout(int variant) {
@@ -272,8 +272,8 @@ constexpr int staged_layout(int variant) {
 
 template <int n, int MODE>
 cudaError_t launch_pairconv_mode(const PairArgs& args, int variant, cudaStream_t stream) {
-  if constexpr (n == 16 && MODE == MODE_APPLY) {
-    if (variant == kWideVariant) return launch_pairconv_wide16(args, stream);
+  if constexpr (n == 16 && (MODE == MODE_APPLY || MODE == MODE_OCC)) {
+    if (variant == kWideVariant) return launch_pairconv_wide16(MODE, args, stream);
   }
   switch (staged_layout<n, MODE>(variant)) {
     case -1:

@@ -270,14 +270,17 @@ __device__ __forceinline__ void wide_scale(float2 (&v)[4][16], const float4* row
   }
 }
 
-// v = conj(a) b with a staged (st) and b in TMEM (128 columns at town); OWN_CONJ: conj(b) a.
-// Warp-wide.
-template <bool OWN_CONJ>
-__device__ __forceinline__ void wide_product(float2 (&v)[4][16], const float4* st, int p0, uint32_t town) {
+// The owner's four pencils from TMEM (128 columns at town).  Warp-wide.
+__device__ __forceinline__ void wide_load_own(float2 (&v)[4][16], uint32_t town) {
 #pragma unroll
   for (int r = 0; r < 4; ++r) tmem_issue_row32(town + (uint32_t)(32 * r), reinterpret_cast<float*>(v[r]));
 #pragma unroll
   for (int r = 0; r < 4; ++r) tmem_wait_ld32(reinterpret_cast<float*>(v[r]));
+}
+
+// v <- conj(a) v with a staged (st); OWN_CONJ: conj(v) a.
+template <bool OWN_CONJ>
+__device__ __forceinline__ void wide_product(float2 (&v)[4][16], const float4* st, int p0) {
 #pragma unroll
   for (int r = 0; r < 4; ++r) {
 #pragma unroll
@@ -484,7 +487,10 @@ __global__ void __launch_bounds__(Wide16::THREADS, 1)
       }
       const float4* st = reinterpret_cast<const float4*>(stage + buf * W::N);
       wide_chain(
-          ga, gb, tw, slot, [&](float2 (&v)[4][16]) { wide_product<false>(v, st, p0, town); },
+          ga, gb, tw, slot, [&](float2 (&v)[4][16]) {
+            wide_load_own(v, town);
+            wide_product<false>(v, st, p0);
+          },
           [&](float2 (&v)[4][16]) { wide_scale(v, row + t, f); },
           [&](float2 (&v)[4][16]) { wide_accumulate<EPI_MUL>(v, st, p0, tacc); });
       // the last warp to finish with this buffer refills it with the partner after next (a
@@ -514,6 +520,215 @@ __global__ void __launch_bounds__(Wide16::THREADS, 1)
     mbar_wait_bounded(&sh.mbar[1], (phases >> 1) & 1u);
   }
   if (active) wide_fold(tacc, sums, t, out, pl.hi, pl.lo, folds == 0, folds == 1, true);
+  tmem_fence_before_sync();
+  __syncthreads();
+  tmem_fence_after_sync();
+  if (warp == 0) tmem_dealloc(tbase, 512);
+}
+
+// The VJP with respect to the occupied orbitals (MODE_OCC) for a tile of four owners u_j at one k':
+// per partner (u_i, ybar_i) the two chains phi = K(conj(u_j) u_i), acc += conj(phi) ybar_i and
+// psi = K(conj(u_j) ybar_i), acc += u_i conj(psi), which differ only in which of the two staged
+// arrays is the factor and which is met at the end.  One stage buffer each: the pairs alternate
+// which chain comes first, so the array that the next pair's first chain starts from is the one
+// this pair has been done with since the start of its second chain, and the other one lands while
+// that first chain is under way.
+//
+// FUSE_W: the omega gradient rides on the transforms (args.vtab2): the first chain keeps its
+// spectrum A and the second adds Re sum_G dv A conj(B), as stage_x_occ does.  A takes the owner's
+// TMEM columns and the owner comes from a copy in the order of the threads (args.spec, one blocked
+// grid a slot), which 32 loads fetch at the start of a chain, when the registers are free for all of
+// them.  Of the 250 us omega costs, those loads are 136, the loads of dv 50 (A in that scratch and the
+// owner in TMEM: 290 us, its loads a few at a time between live spectra).
+// 16^3, 3^3 k, 8 bands: 1,440 us on the pencil-load kernel with omega, 1,383 here; 1,333 and 1,133 us
+// without.
+template <bool FUSE_W>
+__global__ void __launch_bounds__(Wide16::THREADS, 1)
+    pairconv_wide16_occ_kernel(const PairArgs args, const __grid_constant__ CUtensorMap tmap_u,
+                               const __grid_constant__ CUtensorMap tmap_y) {
+  using W = Wide16;
+  extern __shared__ __align__(128) float4 smem4[];
+  __shared__ uint32_t tmem_base_sh;
+  __shared__ uint64_t mbar[2];
+  __shared__ int done[2], fills[2], abort_sh;
+  __shared__ double red[FUSE_W ? W::THREADS : 1];
+  char* sbase = reinterpret_cast<char*>(smem4);
+  sbase += (1024u - (smem_addr_u32(sbase) & 1023u)) & 1023u;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int slot = tid / W::TS, t = tid % W::TS;
+  const WidePlace pl(t);
+  float2* stage = reinterpret_cast<float2*>(sbase);  // [0] u_i, [1] ybar_i
+  float4* row = reinterpret_cast<float4*>(sbase + 2 * W::STAGE_BYTES);
+  float2* g = reinterpret_cast<float2*>(sbase + 2 * W::STAGE_BYTES + W::ROW_BYTES) + slot * W::GRID_CPX;
+  if (tid == 0) {
+    mbar_init(&mbar[0], 1);
+    mbar_init(&mbar[1], 1);
+    done[0] = done[1] = fills[0] = fills[1] = 0;
+    abort_sh = 0;
+    mbar_fence_init();
+  }
+  if (warp == 0) {
+    tmem_alloc(&tmem_base_sh, 512);
+    tmem_relinquish();
+  }
+  const int item = args.item0 + blockIdx.x;
+  const ItemIdx it(args, item);
+  const int band = it.tile * W::SLOTS + slot;
+  const bool active = band < args.n_own;  // uniform over the slot
+  const int nwarps = 2 * min(W::SLOTS, args.n_own - it.tile * W::SLOTS);
+  const int npairs = it.q1 - it.q0, kp_begin = it.q0 / args.n_part;
+  tmem_fence_before_sync();
+  __syncthreads();
+  tmem_fence_after_sync();
+  const uint32_t tbase = tmem_base_sh;
+  const uint32_t tw0 = tbase + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)((warp >> 2) * W::COLS_PER_WARP);
+  const uint32_t tacc = tw0 + W::ACC, town = tw0 + W::OWN;
+  auto fill = [&](int q, int b) {  // one thread
+    ++fills[b];
+    mbar_arrive_expect_tx(&mbar[b], (uint32_t)W::STAGE_BYTES);
+    tensor_copy_2d_g2s(stage + b * W::N, b ? &tmap_y : &tmap_u, 0, (it.q0 + q) * 256, &mbar[b]);
+  };
+  if (tid == 0 && args.inject != 1 && npairs > 0) {
+    fill(0, 0);
+    fill(0, 1);
+  }
+  const size_t oofs = it.split * args.split_stride + ((size_t)it.k * args.n_own + (active ? band : 0)) * W::N;
+  float4* sums = sums_of(args, oofs / W::N, OrbBlk<16>::NBK);
+  float2* out = active ? args.out + oofs : nullptr;
+  // FUSE_W: this thread's 32 float4 of the owner, 64 float4 apart
+  float4* own4 = FUSE_W ? reinterpret_cast<float4*>(args.spec) + ((size_t)blockIdx.x * W::SLOTS + slot) * (W::N / 2) + t : nullptr;
+  if (active) {
+    const float2* own = args.own + ((size_t)it.k * args.n_own + band) * W::N;
+    if constexpr (FUSE_W) {
+#pragma unroll 8
+      for (int i = 0; i < 32; ++i)
+        own4[i * W::TS] = __ldg(reinterpret_cast<const float4*>(own + ((pl.hi + 4 * (i >> 3)) * 16 + pl.lo) * 16) + (i & 7));
+    } else {
+      wide_own_to_tmem(own, pl.hi, pl.lo, town);
+    }
+    float z[32];
+#pragma unroll
+    for (int e = 0; e < 32; ++e) z[e] = 0.f;
+#pragma unroll
+    for (int r = 0; r < 4; ++r) TmemRow<32>::store(tacc + (uint32_t)(32 * r), z);
+  }
+  const WideTw tw(pl.hi);
+  float2* ga = g + wide_a(pl.hi, pl.lo, 0, 0);
+  float2* gb = g + wide_b(pl.hi, pl.lo, 0, 0);
+  const int p0 = pl.hi * 16 + pl.lo;
+  const float f = active ? (float)args.occ[it.k * args.n_occ + band] : 0.f;
+  double wsum = 0.0;
+  const int fspan = fold_span(args.n_part);
+  int folds = 0, cur_kp = -1;
+  const float* dv0 = nullptr;
+  for (int q = 0; q < npairs; ++q) {
+    const int kp = (it.q0 + q) / args.n_part;
+    if (kp != cur_kp) {  // uniform over the CTA
+      const size_t qrow = args.qidx[kp * args.nk_own + it.k];
+      float4 rv[4];
+      wide_row_load(rv, args.vtab + qrow * W::N, args.scale);
+      if (active && cur_kp >= 0 && (kp - kp_begin) / fspan != (cur_kp - kp_begin) / fspan) {
+        wide_fold(tacc, sums, t, out, pl.hi, pl.lo, folds == 0, folds == 1, false);
+        ++folds;
+      }
+      __syncthreads();  // every slot is past its last use of the old row
+      wide_row_store(rv, row);
+      __syncthreads();
+      cur_kp = kp;
+      if (FUSE_W) dv0 = args.vtab2 + qrow * W::N + pl.hi * 256 + pl.lo;  // element (x = k1 + 4 k2, y, z) at (4 k2 16 + y) 16
+    }
+    if (!active) continue;
+    auto wait = [&](int b) {
+      if (!abort_sh && !mbar_wait_bounded(&mbar[b], (uint32_t)q & 1u)) {
+        abort_sh = 1;
+        if (args.status) atomicExch(args.status, kStatusTimeout);
+      }
+    };
+    // the last warp to finish with buffer b refills it with the next partner's array
+    auto release = [&](int b) {
+      __syncwarp();
+      if (lane == 0) {
+        __threadfence_block();
+        if (atomicAdd(&done[b], 1) == nwarps - 1) {
+          done[b] = 0;
+          __threadfence_block();
+          if (q + 1 < npairs && !abort_sh) {
+            fence_proxy_async_smem();
+            fill(q + 1, b);
+          }
+        }
+      }
+    };
+#pragma unroll 1
+    for (int c = 0; c < 2; ++c) {
+      const int b = (q + c) & 1;  // factor; b ^ 1 is met at the end
+      const float4* sp = reinterpret_cast<const float4*>(stage + b * W::N);
+      const float4* se = reinterpret_cast<const float4*>(stage + (b ^ 1) * W::N);
+      if (c == 0) wait(b);
+      wide_chain(
+          ga, gb, tw, slot,
+          [&](float2 (&v)[4][16]) {
+            if constexpr (FUSE_W) {
+#pragma unroll
+              for (int i = 0; i < 32; ++i) {
+                const float4 o = own4[i * W::TS];
+                v[i >> 3][2 * (i & 7)] = make_float2(o.x, o.y);
+                v[i >> 3][2 * (i & 7) + 1] = make_float2(o.z, o.w);
+              }
+            } else {
+              wide_load_own(v, town);
+            }
+            wide_product<true>(v, sp, p0);
+            if (c == 1) release(b);
+          },
+          [&](float2 (&v)[4][16]) {
+            if (FUSE_W && c == 0) {
+#pragma unroll
+              for (int k2 = 0; k2 < 4; ++k2) tmem_put_row32(town + (uint32_t)(32 * k2), reinterpret_cast<const float*>(v[k2]));
+              tmem_wait_st();
+            } else if (FUSE_W) {
+              float d = 0.f;
+#pragma unroll
+              for (int k2 = 0; k2 < 4; ++k2) {
+                float2 a[16];
+                tmem_issue_row32(town + (uint32_t)(32 * k2), reinterpret_cast<float*>(a));
+                float w[16];
+#pragma unroll
+                for (int y = 0; y < 16; ++y) w[y] = __ldg(dv0 + k2 * 1024 + y * 16);
+                tmem_wait_ld32(reinterpret_cast<float*>(a));
+#pragma unroll
+                for (int y = 0; y < 16; ++y) {
+                  const int i = wide_slot(y);
+                  d = fmaf(w[y], fmaf(a[i].x, v[k2][i].x, a[i].y * v[k2][i].y), d);
+                }
+              }
+              wsum += (double)d * (double)(args.scale * f);
+            }
+            wide_scale(v, row + t, f);
+          },
+          [&](float2 (&v)[4][16]) {
+            if (c == 0) wait(b ^ 1);
+            wide_accumulate<EPI_CONJPHI>(v, se, p0, tacc);
+            if (c == 1) release(b ^ 1);
+          });
+    }
+  }
+  __syncthreads();
+  if (tid == 0 && abort_sh) {
+    // a copy may still be in flight after a timeout: give it one more bounded chance to land
+    for (int b = 0; b < 2; ++b)
+      if (fills[b] > 0) mbar_wait_bounded(&mbar[b], (uint32_t)(fills[b] - 1) & 1u);
+  }
+  if (active) wide_fold(tacc, sums, t, out, pl.hi, pl.lo, folds == 0, folds == 1, true);
+  if constexpr (FUSE_W) {  // the item's share of d/d omega, one FP64 partial
+    red[tid] = active ? wsum : 0.0;
+    __syncthreads();
+    if (tid == 0) {
+      double sum = 0.0;
+      for (int e = 0; e < W::THREADS; ++e) sum += red[e];
+      args.partial2[item] = sum;
+    }
+  }
   tmem_fence_before_sync();
   __syncthreads();
   tmem_fence_after_sync();

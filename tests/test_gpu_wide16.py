@@ -38,6 +38,17 @@ def test_wide_apply(nk, n_occ, n_tgt, empty, monkeypatch):
     hse.hse_status(plan)
     ref = oracle.fock_apply(u_occ.astype(np.complex128), occ, u_tgt.astype(np.complex128), kpts, lattice, grid,
                             inputs.OMEGA, inputs.ALPHA)
+    ybar = c64(nk + 3, u_tgt.shape)
+    for omega in (True, False):  # with and without the omega gradient riding on the u_occ pass
+        g_occ, _, g_om = hse.hse_fock_apply_vjp(plan, torch.from_numpy(u_occ).cuda(), torch.from_numpy(occ).cuda(),
+                                                torch.from_numpy(u_tgt).cuda(), torch.from_numpy(ybar).cuda(), need_omega=omega)
+        hse.hse_status(plan)
+        w = [x.astype(np.complex128) for x in (u_occ, u_tgt, ybar)]
+        r_occ, _, r_om = oracle.fock_apply_vjp(w[0], occ, w[1], w[2], kpts, lattice, grid, inputs.OMEGA, inputs.ALPHA)
+        assert np.linalg.norm(g_occ.cpu().numpy() - r_occ) <= 1e-5 * np.linalg.norm(r_occ)
+        if omega:  # a sum of terms of both signs: against its Cauchy-Schwarz scale
+            dvx = oracle.fock_apply(w[0], occ, w[1], kpts, lattice, grid, inputs.OMEGA, inputs.ALPHA, kernel="domega")
+            assert abs(g_om.item() - r_om) <= 1e-5 * np.linalg.norm(w[2]) * np.linalg.norm(dvx)
     got = out.cpu().numpy().astype(np.complex128)
     assert np.linalg.norm(got - ref) <= 1e-5 * np.linalg.norm(ref)
     for k in range(nk):
