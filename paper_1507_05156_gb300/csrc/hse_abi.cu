@@ -306,8 +306,8 @@ struct hse_plan_s {
   bool blocked = true;       // pencil-load launches read pencil-blocked copies (HSE_PENCIL_BLOCKS=0: no)
   int blocks_per_sm = 0;     // fused-kernel variant: 0 default, -1/-2 staged-partner layouts, 1/2/3/5 pencil loads,
                              // kTcVariant the tensor-core form (HSE_C64_TC)
-  bool wide = false;         // the apply runs the two-exchange 16^3 kernel (kWideVariant),
-  bool wide_occ = false;     // and so does the VJP's u_occ pass
+  int apply_variant = 0;     // kernels chosen by estimated time (0: blocks_per_sm): of the apply, kWideVariant or
+  int occ_variant = 0;       // kTwoVariant, and of the VJP's u_occ pass, kWideVariant
   bool tc = false;           // created as HSE_C64_TC (p.dtype then reads HSE_C64)
   int inject = 0;            // test hook (HSE_INJECT_SKIP_FILL=1 at plan creation)
   long long alloc_count = 0;   // device allocations made by this plan so far (plan_malloc)
@@ -476,6 +476,10 @@ double pair_seconds(int n) {
   const double N = (double)n * n * n;
   return (10.0 * N * std::log2(N) + 16.0 * N) / 0.27e12;
 }
+// A pair on an SM: the staged kernel at 18^3 and 20^3, and the two-CTA kernel there.
+double staged_seconds(int n) { return n == 18 ? 3.86e-6 : 4.93e-6; }
+double two_cta_seconds(int n) { return n == 18 ? 3.48e-6 : 4.47e-6; }
+
 // The fused FP64 kernel with T orbitals a CTA: CTAs an SM holds, seconds of an SM a partner takes
 // when they are all busy (6.5 GFLOP/s of the same count; a partial warp costs a whole one, and with
 // one or two CTAs so does a scheduler without a warp in a pass's last round), and seconds a partner
@@ -743,7 +747,9 @@ int hse_plan_create(hse_plan* out, const hse_problem* p) {
   if (const char* env = std::getenv("HSE_BLOCKS_PER_SM")) {
     const int v = std::atoi(env);
     plan->blocks_per_sm = (v < -2 || v > kOneVariant || v == kTcVariant) ? 0 : v;
-    plan->wide = plan->wide_occ = v == kWideVariant && p->dtype == HSE_C64 && p->grid[0] == 16;  // also where it is slower
+    // the kernels that a plan chooses by estimated time, also where they are slower
+    if (p->dtype == HSE_C64 && v == kWideVariant && p->grid[0] == 16) plan->apply_variant = plan->occ_variant = v;
+    if (p->dtype == HSE_C64 && v == kTwoVariant && two_cta_fits(p->grid[0])) plan->apply_variant = v;
   }
   if (plan->tc) plan->blocks_per_sm = kTcVariant;
   const int n1 = p->grid[0], n2 = p->grid[1], n3 = p->grid[2];
@@ -824,16 +830,24 @@ int hse_plan_create(hse_plan* out, const hse_problem* p) {
       const size_t out_bytes = o == ROLE_ENERGY ? 0 : (size_t)k_own[o] * owners[o] * N * sizeof(float2);
       auto tiles = [&](int per) { return (long long)k_own[o] * ((owners[o] + per - 1) / per); };
       SplitChoice choice = choose_split(tiles(T), partners, t_pair, slots, out_bytes, ns_min);
-      if (o == ROLE_TGT && n1 == 16 && plan->blocks_per_sm == 0) {
-        const SplitChoice wide = choose_split(tiles(kWideSlots), partners, kWidePairSeconds, sms, out_bytes, ns_min);
-        plan->wide = plan->wide || wide.seconds < choice.seconds;
-        if (plan->wide) choice = wide;
+      // another kernel of the pass takes it where its estimate is shorter
+      auto consider = [&](int& chosen, int variant, int per, double t_other, long long workers, double extra) {
+        SplitChoice c = choose_split(tiles(per), partners, t_other, workers, out_bytes, ns_min);
+        c.seconds += extra;
+        if (chosen == 0 && c.seconds < choice.seconds) chosen = variant;
+        if (chosen == variant) choice = c;
+      };
+      if (plan->blocks_per_sm == 0 && o == ROLE_TGT && n1 == 16)
+        consider(plan->apply_variant, kWideVariant, kWideSlots, kWidePairSeconds, sms, 0.0);
+      if (plan->blocks_per_sm == 0 && o == ROLE_TGT && two_cta_fits(n1)) {
+        // two CTAs share an SM; the pencil-blocked copies cost two launches and three passes
+        const double copies = 8e-6 + 3.0 * N * sizeof(float2) * ((double)nk * p->n_tgt + (double)nkq * p->n_occ) / 4e12;
+        choice = choose_split(tiles(T), partners, staged_seconds(n1), slots, out_bytes, ns_min);
+        consider(plan->apply_variant, kTwoVariant, T, 2.0 * two_cta_seconds(n1), 2 * sms, copies);
       }
-      if (o == ROLE_OCC && n1 == 16 && plan->blocks_per_sm == 0) {
-        const SplitChoice wide = choose_split(tiles(kWideSlots), partners, kWideOccSeconds, sms, out_bytes, ns_min);
+      if (plan->blocks_per_sm == 0 && o == ROLE_OCC && n1 == 16) {
         choice = choose_split(tiles(T), partners, kPencilOccSeconds16, slots, out_bytes, ns_min);
-        plan->wide_occ = plan->wide_occ || wide.seconds < choice.seconds;
-        if (plan->wide_occ) choice = wide;
+        consider(plan->occ_variant, kWideVariant, kWideSlots, kWideOccSeconds, sms, 0.0);
       }
       int best = choice.ns;
       size_t need = (best > 1 && o != ROLE_ENERGY) ? (size_t)best * k_own[o] * owners[o] * N : 0;
@@ -959,7 +973,9 @@ int hse_plan_create(hse_plan* out, const hse_problem* p) {
                  plan->nsplit[ROLE_TGT], plan->nsplit[ROLE_ENERGY], plan->nsplit[ROLE_OCC],
                  !c64 ? (plan->fused64[ROLE_TGT] ? "fused FP64" : "staged FP64") : (pairconv_c64_pencil_load(n1, MODE_APPLY, plan->blocks_per_sm)
                                              ? (plan->tc ? "pencil-load, tensor-core Y/X" : "pencil-load")
-                                             : plan->wide ? "two-exchange" : "staged-partner"),
+                                             : plan->apply_variant == kWideVariant ? "two-exchange"
+                                             : plan->apply_variant == kTwoVariant  ? "two-CTA pencil-load"
+                                                                                   : "staged-partner"),
                  plan->blocked ? "on" : "off");
   }
   *out = plan;
@@ -1046,9 +1062,10 @@ int to_blocked(hse_plan plan, int mode, PairArgs& a, cudaStream_t st) {
   return cuda_fail(cudaGetLastError());
 }
 
-// Kernel variant of a pass: the plan's, or the two-exchange kernel where it chose that.
+// Kernel variant of a pass: the one chosen for it, or the plan's.
 int kernel_variant(hse_plan plan, int mode) {
-  return (mode == MODE_APPLY && plan->wide) || (mode == MODE_OCC && plan->wide_occ) ? kWideVariant : plan->blocks_per_sm;
+  const int chosen = mode == MODE_APPLY ? plan->apply_variant : mode == MODE_OCC ? plan->occ_variant : 0;
+  return chosen ? chosen : plan->blocks_per_sm;
 }
 
 int run_pairconv(hse_plan plan, int mode, PairArgs a, int n_own, cudaStream_t st) {

@@ -200,6 +200,18 @@ constexpr bool pencil_one_fits() {
   }
 }
 
+// Two-CTA variant (kTwoVariant): the pencil-load kernel with one pencil per thread and two CTAs an
+// SM, for the 18^3 and 20^3 apply.  One CTA's 400 pencils of 20^3 are 13 warps, four on the busiest
+// scheduler where 3.25 are the mean; two CTAs (72 registers a thread) put 7 on it instead of 8, and
+// each fills the other's barriers.  The Z and Y stages of 20^3 synchronise groups of eight x-planes
+// (slab_sync) and its X stage takes the bank-spread order.  A plan takes it for its apply where its
+// estimated time is shorter than the staged kernel's (one CTA an SM, partner by TMA, no blocked
+// copies): 20^3, 64 k, 16 + 16 bands 34.00 -> 30.82 ms (33.0 without the plane groups and the X
+// order, 39.9 with the partner's first read not kept in L1); 18^3, 32 k, 16 + 16 bands 6.66 ->
+// 6.00 ms (6.55 with whole-row TMEM accesses); 20^3, 8 k, 4 + 4 bands 33 against 42 us.
+constexpr int kTwoVariant = 7;
+constexpr bool two_cta_fits(int n) { return n == 18 || n == 20; }
+
 // Staged-partner kernel (pairconv_tma.cuh): one CTA per SM.
 // Encodes the tensor map of a partner array for the staged-partner kernel of side n.
 // swizzle: the 128-byte TMA swizzle (rows of exactly 128 bytes) instead of a padded pitch.
@@ -287,6 +299,9 @@ cudaError_t launch_pairconv_mode(const PairArgs& args, int variant, cudaStream_t
   if constexpr (tc_fits<n, MODE>()) {
     if (variant == kTcVariant) return launch_pairconv_variant<n, MODE, 1, 2, kRaggedThreads, true>(args, stream);
   }
+  if constexpr (two_cta_fits(n) && MODE == MODE_APPLY) {
+    if (variant == kTwoVariant) return launch_pairconv_variant<n, MODE, 2, 1, Geo<n>::NN>(args, stream);
+  }
   if constexpr (pencil_one_fits<n>() && MODE != MODE_OCC) {
     if (variant == kOneVariant || variant <= 0)
       return launch_pairconv_variant<n, MODE, 1, 1, Geo<n>::NN>(args, stream);
@@ -304,6 +319,9 @@ int pairconv_occupancy_mode(int variant) {
   if (staged_layout<n, MODE>(variant) != 0) return 1;
   if constexpr (tc_fits<n, MODE>()) {
     if (variant == kTcVariant) return pairconv_occupancy_variant<n, MODE, 1, 2, kRaggedThreads, true>();
+  }
+  if constexpr (two_cta_fits(n) && MODE == MODE_APPLY) {
+    if (variant == kTwoVariant) return pairconv_occupancy_variant<n, MODE, 2, 1, Geo<n>::NN>();
   }
   if constexpr (pencil_one_fits<n>() && MODE != MODE_OCC) {
     if (variant == kOneVariant || variant <= 0) return pairconv_occupancy_variant<n, MODE, 1, 1, Geo<n>::NN>();

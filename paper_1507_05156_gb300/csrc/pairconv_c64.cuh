@@ -510,19 +510,21 @@ __device__ __forceinline__ void stage_x(float2* g, int t, bool valid, uint32_t t
   for (int ps = 0; ps < PPT; ++ps) {
     if (TS * PPT != G::NN && t + ps * TS >= G::NN) break;
     cpx<float> v[n];
-    if (PPT == 1 && n % 8 == 0 && xs_tab != nullptr) {
+    if (PPT == 1 && n % 4 == 0 && xs_tab != nullptr) {
+      constexpr int C = n % 8 == 0 ? 8 : 4;
       const int xs = xs_tab[t];
       load_s<n, 1>(v, g, xs, G::Q);
       fft<n, -1, float>(v);
 #pragma unroll
-      for (int c = 0; c < n / 8; ++c) {
-        float tv[8];
-        tmem_ld8(ttab + (uint32_t)(8 * c), tv);
+      for (int c = 0; c < n / C; ++c) {
+        float tv[C];
+        if constexpr (C == 8) tmem_ld8(ttab + (uint32_t)(C * c), tv);
+        else tmem_ld4(ttab + (uint32_t)(C * c), tv);
 #pragma unroll
-        for (int e = 0; e < 8; ++e) {
+        for (int e = 0; e < C; ++e) {
           const float w = tv[e] * f;
-          v[8 * c + e].x *= w;
-          v[8 * c + e].y *= w;
+          v[C * c + e].x *= w;
+          v[C * c + e].y *= w;
         }
       }
       fft<n, +1, float>(v);
@@ -648,6 +650,10 @@ __device__ __forceinline__ void stage_z_forward(float2* g, int t, bool valid, co
   }
 }
 
+// Complex values that the one-pencil layout moves between TMEM and registers at a time (0: whole
+// rows).
+__host__ __device__ constexpr int acc_chunk(int n) { return n % 4 == 0 ? 4 : n == 18 ? 6 : 0; }
+
 enum Epi : int {
   EPI_MUL = 0,      // acc += w * phi
   EPI_CONJPHI = 1,  // acc += conj(phi) * w
@@ -684,21 +690,28 @@ __device__ __forceinline__ void stage_z_inverse(const float2* g, int t, const fl
     load_s<n, G::ZVEC>(v, g, pc.zs, 1);
     fft<n, +1, float>(v);
     const uint32_t trow = trow0 + (uint32_t)(ps * G::ROW);
-    if constexpr (PPT == 1 && n % 4 == 0) {
+    if constexpr (PPT == 1 && acc_chunk(n) > 0) {
       // one pencil per thread: the accumulator row and the partner move four complex values
-      // (eight TMEM columns, two 16-byte chunks) at a time, so that only phi stays live
+      // (18^3: six) at a time, so that only phi stays live
+      constexpr int CH = acc_chunk(n);
       const int off = blk ? (p >> 5) * (n / 2) * 32 + (p & 31) : p * (n / 2);
       const float4* w4 = reinterpret_cast<const float4*>(wbase) + off;
 #pragma unroll
-      for (int c = 0; c < n / 4; ++c) {
-        float acc[8];
-        tmem_ld8(trow + (uint32_t)(8 * c), acc);
-        const float4 w0 = blk ? ldg_pol<kLdPartnerLast>(w4 + 32 * (2 * c)) : __ldg(w4 + 2 * c);
-        const float4 w1 = blk ? ldg_pol<kLdPartnerLast>(w4 + 32 * (2 * c + 1)) : __ldg(w4 + 2 * c + 1);
-        const cpx<float> w[4] = {{w0.x, w0.y}, {w0.z, w0.w}, {w1.x, w1.y}, {w1.z, w1.w}};
+      for (int c = 0; c < n / CH; ++c) {
+        float acc[2 * CH];
+        TmemRow<2 * CH>::load(trow + (uint32_t)(2 * CH * c), acc);
+        float4 w[CH / 2];
 #pragma unroll
-        for (int q = 0; q < 4; ++q) epilogue_mac<EPI>(acc[2 * q], acc[2 * q + 1], w[q], v[4 * c + q]);
-        tmem_st8(trow + (uint32_t)(8 * c), acc);
+        for (int q = 0; q < CH / 2; ++q) {
+          const int e = CH / 2 * c + q;
+          w[q] = blk ? ldg_pol<kLdPartnerLast>(w4 + 32 * e) : __ldg(w4 + e);
+        }
+#pragma unroll
+        for (int q = 0; q < CH / 2; ++q) {
+          epilogue_mac<EPI>(acc[4 * q], acc[4 * q + 1], {w[q].x, w[q].y}, v[CH * c + 2 * q]);
+          epilogue_mac<EPI>(acc[4 * q + 2], acc[4 * q + 3], {w[q].z, w[q].w}, v[CH * c + 2 * q + 1]);
+        }
+        TmemRow<2 * CH>::store(trow + (uint32_t)(2 * CH * c), acc);
       }
     } else {
       float acc[G::ROW];
@@ -721,12 +734,17 @@ __device__ __forceinline__ void stage_z_inverse(const float2* g, int t, const fl
 // another between the two CTA-wide barriers around the X stage, so their shared-memory and
 // global-load phases spread out.
 constexpr int gcd_int(int a, int b) { return b == 0 ? a : gcd_int(b, a % b); }
+// 20^3: eight planes (160 threads), and four planes with the idle half warp (96 threads); the
+// barrier takes both counts (kSlab20).
+constexpr int kSlab20 = 160;
 template <int n, int PPT, int TS>
 constexpr int slab_bar_threads() {
   constexpr int L = n / gcd_int(n, 32) * 32;
   if constexpr (PPT == 1 && TS == Geo<n>::NN && Geo<n>::T == 1 && Geo<n>::ZFAST_Y == 1 && Geo<n>::NN % L == 0 &&
                 Geo<n>::NN / L <= 15 && Geo<n>::NN / L > 1) {
     return L;
+  } else if constexpr (n == 20 && PPT == 1) {
+    return kSlab20;
   } else {
     return 0;
   }
@@ -735,7 +753,10 @@ constexpr int slab_bar_threads() {
 // Barrier of the x-slab of thread tid (SB threads; named barrier 1 + tid / SB), or of the CTA.
 template <int SB>
 __device__ __forceinline__ void slab_sync() {
-  if constexpr (SB > 0) {
+  if constexpr (SB == kSlab20) {
+    const int g = (int)threadIdx.x / kSlab20;
+    asm volatile("bar.sync %0, %1;" ::"r"(1 + g), "r"(g == 2 ? 96 : kSlab20) : "memory");
+  } else if constexpr (SB > 0) {
     asm volatile("bar.sync %0, %1;" ::"r"(1 + (int)threadIdx.x / SB), "n"(SB) : "memory");
   } else {
     __syncthreads();
@@ -831,7 +852,7 @@ __device__ __forceinline__ void pairconv_item(const PairArgs& args, int item, fl
   }
   // the bank-spread X-pencil order (x_pencil) of the one-pencil layout, as smem offsets of
   // each thread's X pencil in a table in shared memory (read once per pair, no global lookup)
-  constexpr bool kXTab = PPT == 1 && n % 8 == 0 && !TC && MODE != MODE_OCC && G::T == 1 && G::P != n;
+  constexpr bool kXTab = PPT == 1 && n % 4 == 0 && !TC && MODE != MODE_OCC && G::T == 1 && G::P != n;
   __shared__ unsigned short xs_tab[kXTab ? G::NN : 1];
   if constexpr (kXTab) {
     for (int i = tid; i < G::NN; i += blockDim.x) xs_tab[i] = (unsigned short)Pencil<n>(x_pencil<n, true>(i)).xs;
@@ -852,31 +873,32 @@ __device__ __forceinline__ void pairconv_item(const PairArgs& args, int item, fl
       if (TS * PPT != G::NN && t + ps * TS >= G::NN) break;
       const uint32_t trow = trow0 + (uint32_t)(ps * G::ROW);
       const int p = t + ps * TS;
-      if constexpr (PPT == 1 && n % 4 == 0) {
-        // one pencil per thread: eight accumulator columns (two 16-byte chunks) at a time
+      if constexpr (PPT == 1 && acc_chunk(n) > 0) {
+        constexpr int CH = acc_chunk(n);
         const int loff = blk ? (p >> 5) * (n / 2) * 32 + (p & 31) : p * (n / 2);
         float dpart = 0.f;
 #pragma unroll
-        for (int c = 0; c < n / 4; ++c) {
-          float acc[8];
-          tmem_ld8(trow + (uint32_t)(8 * c), acc);
+        for (int c = 0; c < n / CH; ++c) {
+          float acc[2 * CH];
+          TmemRow<2 * CH>::load(trow + (uint32_t)(2 * CH * c), acc);
           if constexpr (MODE == MODE_APPLY || MODE == MODE_OCC) {
             if (active)
               fold_chunks<n>(acc, sums, p, reinterpret_cast<float4*>(args.out + oofs + (size_t)p * n), first, second,
-                             last, 2 * c, 2);
+                             last, CH / 2 * c, CH / 2);
           } else {
             const float4* l4 = reinterpret_cast<const float4*>(lhs) + loff;
-            const float4 w0 = blk ? ldg_pol<kLdOwner>(l4 + 32 * (2 * c)) : __ldg(l4 + 2 * c);
-            const float4 w1 = blk ? ldg_pol<kLdOwner>(l4 + 32 * (2 * c + 1)) : __ldg(l4 + 2 * c + 1);
-            dpart = fmaf(w0.x, acc[0], fmaf(w0.y, acc[1], dpart));
-            dpart = fmaf(w0.z, acc[2], fmaf(w0.w, acc[3], dpart));
-            dpart = fmaf(w1.x, acc[4], fmaf(w1.y, acc[5], dpart));
-            dpart = fmaf(w1.z, acc[6], fmaf(w1.w, acc[7], dpart));
+#pragma unroll
+            for (int q = 0; q < CH / 2; ++q) {
+              const int e = CH / 2 * c + q;
+              const float4 w = blk ? ldg_pol<kLdOwner>(l4 + 32 * e) : __ldg(l4 + e);
+              dpart = fmaf(w.x, acc[4 * q], fmaf(w.y, acc[4 * q + 1], dpart));
+              dpart = fmaf(w.z, acc[4 * q + 2], fmaf(w.w, acc[4 * q + 3], dpart));
+            }
           }
           if (!last) {
 #pragma unroll
-            for (int e = 0; e < 8; ++e) acc[e] = 0.f;
-            tmem_st8(trow + (uint32_t)(8 * c), acc);
+            for (int e = 0; e < 2 * CH; ++e) acc[e] = 0.f;
+            TmemRow<2 * CH>::store(trow + (uint32_t)(2 * CH * c), acc);
           }
         }
         if constexpr (MODE == MODE_ENERGY || MODE == MODE_DOT) dsum += (double)dpart;
