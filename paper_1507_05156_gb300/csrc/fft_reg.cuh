@@ -149,14 +149,16 @@ struct Butterfly<4, DIR, T> {
 };
 
 // 32 operations: the cosine sums through t1 + t2 and t1 - t2 (c1 + c2 = -1/2, c1 - c2 = sqrt(5)/2),
-// the sine sums as s1 (t3 + r t4) and s1 (r t3 - t4), r = s2 / s1, with the factor s1 in the last
-// multiply-adds (36 with the four products written out).
+// the sine sums as s2 (g t3 + t4) and s2 (t3 - g t4), g = s1 / s2, with the factor s2 in the last
+// multiply-adds (36 with the four products written out).  Rounded to FP32, s2 and g change a plane
+// wave by 6e-10 through a transform and its inverse; s1 and s2 / s1 would by 4e-8, the four sines
+// and cosines by 2e-8.
 template <int DIR, typename T>
 struct Butterfly<5, DIR, T> {
   static __host__ __device__ __forceinline__ void run(cpx<T>* a) {
     constexpr T hr5 = T(0.559016994374947424102293417182819059);  // sqrt(5) / 4
-    constexpr T s1 = T(DIR * trig2pi(1, 5, 1));
-    constexpr T r = T(trig2pi(2, 5, 1) / trig2pi(1, 5, 1));
+    constexpr T s2 = T(DIR * trig2pi(2, 5, 1));
+    constexpr T g = T(trig2pi(1, 5, 1) / trig2pi(2, 5, 1));
     const cpx<T> t1 = cadd(a[1], a[4]);
     const cpx<T> t2 = cadd(a[2], a[3]);
     const cpx<T> t3 = csub(a[1], a[4]);
@@ -165,13 +167,13 @@ struct Butterfly<5, DIR, T> {
     const cpx<T> m = {a[0].x - T(0.25) * t.x, a[0].y - T(0.25) * t.y};
     const cpx<T> p1 = {m.x + hr5 * u.x, m.y + hr5 * u.y};
     const cpx<T> p2 = {m.x - hr5 * u.x, m.y - hr5 * u.y};
-    const cpx<T> q1 = {t3.x + r * t4.x, t3.y + r * t4.y};
-    const cpx<T> q2 = {r * t3.x - t4.x, r * t3.y - t4.y};
+    const cpx<T> q1 = {g * t3.x + t4.x, g * t3.y + t4.y};
+    const cpx<T> q2 = {t3.x - g * t4.x, t3.y - g * t4.y};
     a[0] = cadd(a[0], t);
-    a[1] = {p1.x - s1 * q1.y, p1.y + s1 * q1.x};
-    a[4] = {p1.x + s1 * q1.y, p1.y - s1 * q1.x};
-    a[2] = {p2.x - s1 * q2.y, p2.y + s1 * q2.x};
-    a[3] = {p2.x + s1 * q2.y, p2.y - s1 * q2.x};
+    a[1] = {p1.x - s2 * q1.y, p1.y + s2 * q1.x};
+    a[4] = {p1.x + s2 * q1.y, p1.y - s2 * q1.x};
+    a[2] = {p2.x - s2 * q2.y, p2.y + s2 * q2.x};
+    a[3] = {p2.x + s2 * q2.y, p2.y - s2 * q2.x};
   }
 };
 
