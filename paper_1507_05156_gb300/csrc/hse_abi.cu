@@ -318,8 +318,8 @@ struct hse_plan_s {
   float2* split_buf = nullptr;  // [nsplit][nk_own][n_own][N] partial outputs when nsplit > 1
   size_t split_buf_elems = 0;
   float2* comp_buf = nullptr;   // [nsplit][nk_own][n_own][2][blocked] running sums s, c (APPLY / OCC)
-  // pencil-blocked copies of the orbital arrays a pencil-load launch reads (allocated on first
-  // use, grown when a larger call comes)
+  // pencil-blocked copies of the orbital arrays a pencil-load launch reads (allocated with the plan
+  // for a two-CTA apply, else on first use and grown when a larger call comes)
   float2* blk_buf = nullptr;
   size_t blk_elems = 0;
   // MODE_OCC with the omega gradient fused in (allocated on first use): per CTA of a launch
@@ -478,9 +478,13 @@ double pair_seconds(int n) {
   const double N = (double)n * n * n;
   return (10.0 * N * std::log2(N) + 16.0 * N) / 0.27e12;
 }
-// A pair on an SM: the staged kernel at 18^3 and 20^3, and the two-CTA kernel there.
-double staged_seconds(int n) { return n == 18 ? 3.86e-6 : 4.93e-6; }
-double two_cta_seconds(int n) { return n == 18 ? 3.48e-6 : 4.47e-6; }
+// A partner of an owner tile on an SM: the staged kernel and the two-CTA kernel.
+double staged_seconds(int n) {
+  return n == 8 ? 2.06e-6 : n == 10 ? 2.64e-6 : n == 12 ? 3.85e-6 : n == 18 ? 3.86e-6 : 4.93e-6;
+}
+double two_cta_seconds(int n) {
+  return n == 8 ? 1.91e-6 : n == 10 ? 2.15e-6 : n == 12 ? 3.52e-6 : n == 18 ? 3.48e-6 : 4.47e-6;
+}
 
 // The fused FP64 kernel with T orbitals a CTA: CTAs an SM holds, seconds of an SM a partner takes
 // when they are all busy (6.5 GFLOP/s of the same count; a partial warp costs a whole one, and with
@@ -866,6 +870,13 @@ int hse_plan_create(hse_plan* out, const hse_problem* p) {
       plan->split_buf_elems = buf;
     }
     HSE_TRY(plan_malloc(plan, &plan->comp_buf, comp * sizeof(float2)));
+    if (plan->apply_variant == kTwoVariant && plan->blocked) {
+      // the blocked copies of every pass, so that no call of the plan allocates or moves them: the
+      // first apply can be captured into a graph, and a later pass leaves that graph's copies in place
+      const size_t own = (size_t)nk * p->n_tgt, occ = (size_t)nkq * p->n_occ;
+      plan->blk_elems = std::max(2 * own + occ, (size_t)nk * p->n_occ + occ) * blocked_stride(n1);
+      HSE_TRY(plan_malloc(plan, &plan->blk_buf, plan->blk_elems * sizeof(float2)));
+    }
   }
   size_t e64_items = 0;
   if (plan->p.dtype == HSE_C128 && f64_grid_bytes(n1, n2, n3) <= kF64MaxSmem) {

@@ -201,16 +201,17 @@ constexpr bool pencil_one_fits() {
 }
 
 // Two-CTA variant (kTwoVariant): the pencil-load kernel with one pencil per thread and two CTAs an
-// SM, for the 18^3 and 20^3 apply.  One CTA's 400 pencils of 20^3 are 13 warps, four on the busiest
+// SM, for the apply of most sides.  One CTA's 400 pencils of 20^3 are 13 warps, four on the busiest
 // scheduler where 3.25 are the mean; two CTAs (72 registers a thread) put 7 on it instead of 8, and
 // each fills the other's barriers.  The Z and Y stages of 20^3 synchronise groups of eight x-planes
 // (slab_sync) and its X stage takes the bank-spread order.  A plan takes it for its apply where its
 // estimated time is shorter than the staged kernel's (one CTA an SM, partner by TMA, no blocked
 // copies): 20^3, 64 k, 16 + 16 bands 34.00 -> 30.82 ms (33.0 without the plane groups and the X
 // order, 39.9 with the partner's first read not kept in L1); 18^3, 32 k, 16 + 16 bands 6.66 ->
-// 6.00 ms (6.55 with whole-row TMEM accesses); 20^3, 8 k, 4 + 4 bands 33 against 42 us.
+// 6.00 ms (6.55 with whole-row TMEM accesses); 20^3, 4 k, 4 + 4 bands 33 against 42 us.  64 k, 16 + 16
+// bands: 12^3 6.64 -> 6.06 ms, 10^3 4.55 -> 3.70 ms, 8^3 1.778 -> 1.645 ms (several owners a CTA there).
 constexpr int kTwoVariant = 7;
-constexpr bool two_cta_fits(int n) { return n == 18 || n == 20; }
+constexpr bool two_cta_fits(int n) { return n == 8 || n == 10 || n == 12 || n == 18 || n == 20; }
 
 // Staged-partner kernel (pairconv_tma.cuh): one CTA per SM.
 // Encodes the tensor map of a partner array for the staged-partner kernel of side n.

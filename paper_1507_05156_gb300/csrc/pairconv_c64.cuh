@@ -739,6 +739,8 @@ constexpr int gcd_int(int a, int b) { return b == 0 ? a : gcd_int(b, a % b); }
 constexpr int kSlab20 = 160;
 template <int n, int PPT, int TS>
 constexpr int slab_bar_threads() {
+  // 8^3: the 32 pencils of a warp are whole planes of one owner slot, __syncwarp is enough
+  if constexpr (PPT == 1 && 32 % n == 0 && TS % 32 == 0 && Geo<n>::ZFAST_Y == 1) return 32;
   constexpr int L = n / gcd_int(n, 32) * 32;
   if constexpr (PPT == 1 && TS == Geo<n>::NN && Geo<n>::T == 1 && Geo<n>::ZFAST_Y == 1 && Geo<n>::NN % L == 0 &&
                 Geo<n>::NN / L <= 15 && Geo<n>::NN / L > 1) {
@@ -753,7 +755,9 @@ constexpr int slab_bar_threads() {
 // Barrier of the x-slab of thread tid (SB threads; named barrier 1 + tid / SB), or of the CTA.
 template <int SB>
 __device__ __forceinline__ void slab_sync() {
-  if constexpr (SB == kSlab20) {
+  if constexpr (SB == 32) {
+    __syncwarp();
+  } else if constexpr (SB == kSlab20) {
     const int g = (int)threadIdx.x / kSlab20;
     asm volatile("bar.sync %0, %1;" ::"r"(1 + g), "r"(g == 2 ? 96 : kSlab20) : "memory");
   } else if constexpr (SB > 0) {
