@@ -56,7 +56,7 @@ extern "C" {
 
 /* Arithmetic of the pair convolutions. */
 #define HSE_C64   0  /* complex64 orbitals, fused FP32 kernel, FP64 energy/omega reduction */
-#define HSE_C128  1  /* complex128 orbitals, plain staged FP64 kernels                     */
+#define HSE_C128  1  /* complex128 orbitals, fused or staged FP64 kernels                  */
 /* complex64 orbitals (as HSE_C64), the Y and X axis transforms of V_x u and E_x as split-FP16
  * tensor-core GEMMs (hi/lo halves, three products, FP32 accumulation), the Z transforms and
  * every other step as HSE_C64; 24^3 grids only (else HSE_ERR_UNSUPPORTED_GRID).  The VJP's
@@ -268,18 +268,20 @@ int hse_current(hse_plan plan, const void *psi, const double *occ, const double 
  * Asynchronous on `stream`.  Not for batched plans. */
 int hse_overlap(hse_plan plan, const void *u, int nbands, double *S, hse_stream_t stream);
 
-/* Orthonormalises the bands of every k-point in place, in band order: modified Gram-Schmidt
- * (band a loses its component along each earlier band b < a in turn, then is divided by its
- * norm), applied twice, with every inner product and update in FP64.  complex64 orbitals are
- * widened into an FP64 copy and rounded once when written back; complex128 ones are updated
- * in place.  A band that is linearly dependent on the earlier ones (its norm after the
+/* Orthonormalises the bands of every k-point in place, in band order (Gram-Schmidt: band a
+ * loses its component along each earlier band b < a, then is divided by its norm), with every
+ * inner product and update in FP64.  Up to 64 bands that are well conditioned go through the
+ * Cholesky factor of their overlap matrix (complex128: twice); the others, and a few small
+ * bands, through modified Gram-Schmidt applied twice (complex64 ones in an FP64 copy).
+ * complex64 bands are rounded once, when written back.  A band that is linearly dependent on the earlier ones (its norm after the
  * projections at most 1e-12 of its norm before them for complex128, 1e-5 for complex64, whose
  * rounding leaves about 1e-7 of any band outside the span of the others) is set to zero and
  * the plan's status word records HSE_ERR_SINGULAR (returned by hse_status).
  *   u  device [nk][nbands][N] (the plan's dtype), 1 <= nbands <= 4096, overwritten
  * complex64: the first call (or one with more bands than before) allocates an FP64 copy of
- * the orbitals in the plan (device-wide synchronisation).  Asynchronous on `stream`
- * otherwise.  Not for batched plans. */
+ * the orbitals in the plan (device-wide synchronisation); either type allocates the overlap
+ * matrices and factors, except a complex128 call captured into a graph, which takes
+ * Gram-Schmidt.  Asynchronous on `stream` otherwise.  Not for batched plans. */
 int hse_orthonormalize(hse_plan plan, void *u, int nbands, hse_stream_t stream);
 
 #ifdef __cplusplus

@@ -1751,17 +1751,27 @@ int hse_orthonormalize(hse_plan plan, void* u, int nbands, hse_stream_t stream) 
     if (e != cudaSuccess) return cuda_fail(e);
     plan->ortho_elems = count;
   }
-  const size_t scratch = ortho_scratch_bytes(p.nk, nbands);
+  // Without scratch the Gram-Schmidt kernel does it all: a captured complex128 call, so that nothing
+  // is allocated while capturing and no graph holds scratch that a larger call would move; and any
+  // call for which there is no memory.
+  cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+  const bool capturing = p.dtype == HSE_C128 && (cudaStreamIsCapturing(S(stream), &capture) != cudaSuccess ||
+                                                 capture != cudaStreamCaptureStatusNone);
+  size_t scratch = capturing ? 0 : ortho_scratch_bytes(p.nk, nbands);
   if (scratch > plan->ortho_scratch_size) {
     cudaFree(plan->ortho_scratch);
     plan->ortho_scratch = nullptr;
     plan->ortho_scratch_size = 0;
     const cudaError_t e = plan_malloc(plan, &plan->ortho_scratch, scratch);
-    if (e != cudaSuccess) return cuda_fail(e);
+    if (e != cudaSuccess && e != cudaErrorMemoryAllocation) return cuda_fail(e);
+    if (e != cudaSuccess) {
+      cudaGetLastError();
+      scratch = 0;
+    }
     plan->ortho_scratch_size = scratch;
   }
   return cuda_fail(launch_orthonormalize(p.dtype == HSE_C128, u, p.nk, nbands, plan->N, plan->dV, plan->ortho_work,
-                                         plan->ortho_scratch, plan->status, S(stream)));
+                                         scratch ? plan->ortho_scratch : nullptr, plan->status, S(stream)));
 }
 
 int hse_hartree_potential(hse_plan plan, const void* psi, const double* occ, double* vh, hse_stream_t stream) {

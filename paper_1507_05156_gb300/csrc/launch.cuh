@@ -44,8 +44,8 @@ constexpr int kStatusSingular = -8;  // HSE_ERR_SINGULAR
 cudaError_t launch_overlap(bool c128, const void* u, int nk, int nb, size_t N, double dV, double2* S,
                            cudaStream_t stream);
 // u [nk][nb][N] in place (two modified Gram-Schmidt passes, or their equal); work: [nk][nb][N]
-// double2 scratch for complex64 orbitals (unused for complex128); scratch: ortho_scratch_bytes;
-// status: the plan's status word.
+// double2 scratch for complex64 orbitals (unused for complex128); scratch: ortho_scratch_bytes, or
+// null (Gram-Schmidt only); status: the plan's status word.
 size_t ortho_scratch_bytes(int nk, int nb);
 cudaError_t launch_orthonormalize(bool c128, void* u, int nk, int nb, size_t N, double dV, double2* work, void* scratch,
                                   int* status, cudaStream_t stream);

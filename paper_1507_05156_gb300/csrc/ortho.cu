@@ -445,7 +445,7 @@ cudaError_t orthonormalize(C* u, int nk, int nb, size_t N, double dV, double2* w
   // 3.4 us (2 + N / 1024) nb (nb + 1) in each wave of k-points (16^3, 8 k, 1 band, complex128: 41
   // against 73 us).
   const double sweeps = 3.4 * nb * (nb + 1.0) * (2.0 + N / 1024.0) * ((nk + 607) / 608);
-  if (ortho_scratch_bytes(nk, nb) && sweeps > (kC128 ? 75.0 : 40.0)) {
+  if (scratch && sweeps > (kC128 ? 75.0 : 40.0)) {
     double2* S = static_cast<double2*>(scratch);
     double2* T = S + (size_t)nk * nb * nb;
     skip = reinterpret_cast<int*>(T + (size_t)nk * nb * nb);

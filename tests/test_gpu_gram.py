@@ -51,3 +51,23 @@ def test_overlap_and_orthonormalize(n, nk, nb, dtype):
     for k in range(nk):
         err = np.linalg.norm((got[k] - q[k]).reshape(nb, -1), axis=1) / np.linalg.norm(q[k].reshape(nb, -1), axis=1)
         assert err.max() <= tol * (cond if k == nk - 1 else 1.0)
+
+
+def test_first_complex128_call_is_captured():
+    """A plan's first complex128 call, captured into a graph, allocates nothing; a call with more bands
+    in between does not disturb its replay."""
+    n, nk, nb = 12, 2, 6
+    plan, dV = _plan((n, n, n), nk, nb, torch.complex128)
+    u = inputs.random_orbitals(7, (nk, nb, n, n, n)) * 0.05
+    d = torch.from_numpy(u).cuda()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        hse.hse_orthonormalize(plan, d)
+    big = torch.from_numpy(inputs.random_orbitals(8, (nk, 2 * nb, n, n, n)) * 0.05).cuda()
+    hse.hse_orthonormalize(plan, big)
+    d.copy_(torch.from_numpy(u))
+    graph.replay()
+    hse.hse_status(plan)
+    q = oracle.ortho.gram_schmidt(u, dV)
+    err = np.linalg.norm((d.cpu().numpy() - q).reshape(nk * nb, -1), axis=1) / np.linalg.norm(q.reshape(nk * nb, -1), axis=1)
+    assert err.max() <= 1e-12
