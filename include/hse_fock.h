@@ -114,9 +114,10 @@ int hse_plan_destroy(hse_plan plan);
  * terms are summed over the bands of each k' in FP32 and over k' with compensation (TwoSum).
  * Asynchronous on `stream`, except
  * that a complex64 call running the pencil-load kernel (24^3 grids here, and the VJP with
- * respect to u_occ at every size) copies the orbitals it reads into plan scratch in a
+ * respect to u_occ at most sizes) copies the orbitals it reads into plan scratch in a
  * pencil-blocked layout, which the first such call (or one needing more than before)
- * allocates with device-wide synchronisation. */
+ * allocates with device-wide synchronisation; plans whose apply runs that kernel at 8^3 to
+ * 20^3 hold the copies from their creation. */
 int hse_fock_apply(hse_plan plan, const void *u_occ, const double *occ, const void *u_tgt,
                    void *vx_out, hse_stream_t stream);
 
