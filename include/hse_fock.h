@@ -280,9 +280,11 @@ int hse_overlap(hse_plan plan, const void *u, int nbands, double *S, hse_stream_
  * the plan's status word records HSE_ERR_SINGULAR (returned by hse_status).
  *   u  device [nk][nbands][N] (the plan's dtype), 1 <= nbands <= 4096, overwritten
  * complex64: the first call (or one with more bands than before) allocates an FP64 copy of
- * the orbitals in the plan (device-wide synchronisation); either type allocates the overlap
- * matrices and factors, except a complex128 call captured into a graph, which takes
- * Gram-Schmidt.  Asynchronous on `stream` otherwise.  Not for batched plans. */
+ * the orbitals and their overlap matrices and factors in the plan (device-wide
+ * synchronisation).  complex128: a stream's first call (or one with more bands than before)
+ * allocates matrices and factors for that stream; a call captured into a graph allocates
+ * nothing and takes Gram-Schmidt, and calls on several streams may overlap.  Asynchronous on
+ * `stream` otherwise.  Not for batched plans. */
 int hse_orthonormalize(hse_plan plan, void *u, int nbands, hse_stream_t stream);
 
 #ifdef __cplusplus

@@ -24,6 +24,7 @@
 #include <cstdlib>
 #include <cstring>
 #include <map>
+#include <mutex>
 #include <new>
 #include <string>
 #include <vector>
@@ -343,8 +344,15 @@ struct hse_plan_s {
   double2* hart_work = nullptr;   // Hartree potential: [N] FP64 transform
   double2* ortho_work = nullptr;  // orthonormalisation of complex64 orbitals: FP64 copy
   size_t ortho_elems = 0;
-  void* ortho_scratch = nullptr;  // overlap matrices, factors and flags of the orthonormalisation
+  void* ortho_scratch = nullptr;  // overlap matrices, factors and flags of the orthonormalisation (complex64)
   size_t ortho_scratch_size = 0;
+  struct OrthoBlock {  // the same for complex128 calls on one stream
+    unsigned long long stream;  // cudaStreamGetId
+    size_t bytes;
+    void* p;
+  };
+  std::vector<OrthoBlock> ortho_blocks;  // kept until the plan goes
+  std::mutex ortho_mutex;
   // batched plans (hse_plan_create_batched)
   bool batched = false;
   std::vector<hse_plan> cells;          // one sub-plan (kernel tables) per cell
@@ -580,6 +588,39 @@ long long fail_alloc_from_env() {
   return env ? std::atoll(env) : -1;
 }
 
+// Scratch of a complex128 orthonormalisation of nbands on stream st, or null: the caller then takes
+// Gram-Schmidt.  Null while st is captured (nothing is allocated into a capture, no graph holds plan
+// memory), where there is no memory, and past kOrthoBlocks blocks.  A block serves its stream alone and
+// is not moved; a call with more bands gets another, of the next power of two of bands.
+constexpr size_t kOrthoBlocks = 16;
+void* ortho_block(hse_plan plan, int nbands, cudaStream_t st) {
+  cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+  unsigned long long id = 0;
+  if (cudaStreamIsCapturing(st, &capture) != cudaSuccess || capture != cudaStreamCaptureStatusNone ||
+      cudaStreamGetId(st, &id) != cudaSuccess) {
+    cudaGetLastError();  // of a refused query: not the launches' error
+    return nullptr;
+  }
+  const size_t need = ortho_scratch_bytes(plan->p.nk, nbands);
+  for (const auto& b : plan->ortho_blocks)
+    if (b.stream == id && b.bytes >= need) return b.p;
+  if (plan->ortho_blocks.size() >= kOrthoBlocks) return nullptr;
+  int cap = 4;
+  while (cap < nbands) cap *= 2;
+  hse_plan_s::OrthoBlock b{id, ortho_scratch_bytes(plan->p.nk, cap), nullptr};
+  // a capture on another stream or thread goes on undisturbed
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  cudaThreadExchangeStreamCaptureMode(&mode);
+  const cudaError_t e = plan_malloc(plan, &b.p, b.bytes);
+  cudaThreadExchangeStreamCaptureMode(&mode);
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    return nullptr;
+  }
+  plan->ortho_blocks.push_back(b);
+  return b.p;
+}
+
 bool invert3(const double* A, double* inv) {
   const double det = A[0] * (A[4] * A[8] - A[5] * A[7]) - A[1] * (A[3] * A[8] - A[5] * A[6]) + A[2] * (A[3] * A[7] - A[4] * A[6]);
   if (!(std::fabs(det) > 1e-12) || !std::isfinite(det)) return false;
@@ -711,6 +752,7 @@ int hse_plan_destroy(hse_plan plan) {
   cudaFree(plan->cur_partial);
   cudaFree(plan->hart_work);
   cudaFree(plan->ortho_scratch);
+  for (const auto& b : plan->ortho_blocks) cudaFree(b.p);
   cudaFree(plan->ortho_work);
   cudaSetDevice(prev);
   delete plan;
@@ -1743,35 +1785,34 @@ int hse_orthonormalize(hse_plan plan, void* u, int nbands, hse_stream_t stream) 
   if (!aligned16(u)) return HSE_ERR_INVALID_ARG;
   const hse_problem& p = plan->p;
   const size_t count = (size_t)p.nk * nbands * plan->N;
-  if (p.dtype == HSE_C64 && count > plan->ortho_elems) {
-    cudaFree(plan->ortho_work);
-    plan->ortho_work = nullptr;
-    plan->ortho_elems = 0;
-    const cudaError_t e = plan_malloc(plan, &plan->ortho_work, count * sizeof(double2));
-    if (e != cudaSuccess) return cuda_fail(e);
-    plan->ortho_elems = count;
-  }
-  // Without scratch the Gram-Schmidt kernel does it all: a captured complex128 call, so that nothing
-  // is allocated while capturing and no graph holds scratch that a larger call would move; and any
-  // call for which there is no memory.
-  cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
-  const bool capturing = p.dtype == HSE_C128 && (cudaStreamIsCapturing(S(stream), &capture) != cudaSuccess ||
-                                                 capture != cudaStreamCaptureStatusNone);
-  size_t scratch = capturing ? 0 : ortho_scratch_bytes(p.nk, nbands);
-  if (scratch > plan->ortho_scratch_size) {
-    cudaFree(plan->ortho_scratch);
-    plan->ortho_scratch = nullptr;
-    plan->ortho_scratch_size = 0;
-    const cudaError_t e = plan_malloc(plan, &plan->ortho_scratch, scratch);
-    if (e != cudaSuccess && e != cudaErrorMemoryAllocation) return cuda_fail(e);
-    if (e != cudaSuccess) {
-      cudaGetLastError();
-      scratch = 0;
+  const size_t need = ortho_scratch_bytes(p.nk, nbands);
+  if (p.dtype == HSE_C64) {
+    // The factors' scratch goes with the FP64 copy, for as many bands as that holds, so that it moves
+    // only where the copy does: in a call with more bands than before.
+    if (count > plan->ortho_elems) {
+      cudaFree(plan->ortho_work);
+      cudaFree(plan->ortho_scratch);
+      plan->ortho_work = nullptr;
+      plan->ortho_scratch = nullptr;
+      plan->ortho_elems = plan->ortho_scratch_size = 0;
+      cudaError_t e = plan_malloc(plan, &plan->ortho_work, count * sizeof(double2));
+      if (e != cudaSuccess) return cuda_fail(e);
+      plan->ortho_elems = count;
+      const size_t bytes = ortho_scratch_bytes(p.nk, std::min(nbands, kGramBands));
+      e = bytes ? plan_malloc(plan, &plan->ortho_scratch, bytes) : cudaSuccess;
+      if (e == cudaSuccess) plan->ortho_scratch_size = bytes;
+      else if (e == cudaErrorMemoryAllocation) cudaGetLastError();  // Gram-Schmidt does it all
+      else return cuda_fail(e);
     }
-    plan->ortho_scratch_size = scratch;
+    return cuda_fail(launch_orthonormalize(false, u, p.nk, nbands, plan->N, plan->dV, plan->ortho_work,
+                                           need && need <= plan->ortho_scratch_size ? plan->ortho_scratch : nullptr,
+                                           plan->status, S(stream)));
   }
-  return cuda_fail(launch_orthonormalize(p.dtype == HSE_C128, u, p.nk, nbands, plan->N, plan->dV, plan->ortho_work,
-                                         scratch ? plan->ortho_scratch : nullptr, plan->status, S(stream)));
+  // complex128 orbitals need no scratch for Gram-Schmidt, so calls of several streams and host threads
+  // may overlap: the factors' scratch belongs to one stream, and a call holds the lock over its launches.
+  std::lock_guard<std::mutex> lock(plan->ortho_mutex);
+  return cuda_fail(launch_orthonormalize(true, u, p.nk, nbands, plan->N, plan->dV, nullptr,
+                                         need ? ortho_block(plan, nbands, S(stream)) : nullptr, plan->status, S(stream)));
 }
 
 int hse_hartree_potential(hse_plan plan, const void* psi, const double* occ, double* vh, hse_stream_t stream) {

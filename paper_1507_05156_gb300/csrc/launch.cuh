@@ -40,6 +40,7 @@ cudaError_t launch_current(bool c128, const void* psi, const double* occ, const 
 
 // Overlap matrices and Gram-Schmidt orthonormalisation in FP64 (ortho.cu).
 constexpr int kStatusSingular = -8;  // HSE_ERR_SINGULAR
+constexpr int kGramBands = 64;       // most bands of the tiled kernels
 // S device [nk][nb][nb] double2: S[k][a][b] = dV sum_r conj(u_{a,k}) u_{b,k}
 cudaError_t launch_overlap(bool c128, const void* u, int nk, int nb, size_t N, double dV, double2* S,
                            cudaStream_t stream);

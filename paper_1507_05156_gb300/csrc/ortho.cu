@@ -89,7 +89,6 @@ __global__ void __launch_bounds__(kOverlapThreads) overlap_kernel(const C* __res
   }
 }
 
-constexpr int kGramBands = 64;   // most bands of the tiled kernels
 constexpr int kGramTiles = 10;   // 4 x 4 band tiles (one warp each) per CTA: all of 16 bands
 
 // One grid point's products of a tile: acc[i][j] += conj(x_i) y_j.  DIAG: j >= i only, and the real
