@@ -125,17 +125,30 @@ __global__ void reduce_splits_f64(double2* __restrict__ out, const double2* __re
 static std::atomic<uint64_t> g_launches{0};
 constexpr int kMaxBatchSplit = 4;
 
-// The CUDA driver API's tensor-map encoder, obtained through the runtime (no link against libcuda).
+// Entry point of the CUDA driver API, obtained through the runtime (no link against libcuda).
+template <class F>
+F driver_entry(const char* name, int version) {
+  void* fn = nullptr;
+  cudaDriverEntryPointQueryResult q = cudaDriverEntryPointSymbolNotFound;
+  return cudaGetDriverEntryPointByVersion(name, &fn, version, cudaEnableDefault, &q) == cudaSuccess &&
+                 q == cudaDriverEntryPointSuccess
+             ? (F)fn
+             : nullptr;
+}
+
+// The tensor-map encoder needs a current context, and a host thread whose first CUDA work this is (an
+// autograd thread, say) has none yet: the runtime binds its device's.  A context that is current stays.
 cudaError_t make_partner_tmap(CUtensorMap* map, const void* base, int n, long long rows, int sp, int box_rows,
                               bool swizzle) {
-  static PFN_cuTensorMapEncodeTiled_v12000 encode = nullptr;
-  if (!encode) {
-    void* fn = nullptr;
-    cudaDriverEntryPointQueryResult q = cudaDriverEntryPointSymbolNotFound;
-    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &q) != cudaSuccess ||
-        q != cudaDriverEntryPointSuccess || !fn)
-      return cudaErrorNotSupported;
-    encode = (PFN_cuTensorMapEncodeTiled_v12000)fn;
+  static const auto encode = driver_entry<PFN_cuTensorMapEncodeTiled_v12000>("cuTensorMapEncodeTiled", 12000);
+  static const auto current = driver_entry<PFN_cuCtxGetCurrent_v4000>("cuCtxGetCurrent", 4000);
+  if (!encode || !current) return cudaErrorNotSupported;
+  CUcontext ctx = nullptr;
+  if (current(&ctx) != CUDA_SUCCESS || !ctx) {
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaSetDevice(dev);
+    if (e != cudaSuccess) return e;
   }
   if (rows <= 0 || rows > ((long long)1 << 32)) return cudaErrorInvalidValue;
   const cuuint64_t dims[2] = {(cuuint64_t)(2 * n), (cuuint64_t)rows};  // floats of a pencil, pencils
