@@ -333,7 +333,7 @@ struct hse_plan_s {
   size_t split_buf_elems = 0;
   float2* comp_buf = nullptr;   // [nsplit][nk_own][n_own][2][blocked] running sums s, c (APPLY / OCC)
   // pencil-blocked copies of the orbital arrays a pencil-load launch reads (allocated with the plan
-  // for a two-CTA apply, else on first use and grown when a larger call comes)
+  // for a two-CTA apply of a plan of its own, else on first use and grown when a larger call comes)
   float2* blk_buf = nullptr;
   size_t blk_elems = 0;
   // MODE_OCC with the omega gradient fused in (allocated on first use): per CTA of a launch
@@ -772,8 +772,9 @@ int hse_plan_destroy(hse_plan plan) {
   return HSE_OK;
 }
 
-int hse_plan_create(hse_plan* out, const hse_problem* p) {
-  const NvtxRange nvtx_range("hse_plan_create");
+// lone: a plan of its own, which holds the copies of a two-CTA apply from the start (a batched plan's
+// cells may run in another form and make them on first use).
+static int create_plan(hse_plan* out, const hse_problem* p, bool lone) {
   if (!out) return HSE_ERR_INVALID_ARG;
   *out = nullptr;
   int rc = validate_problem(p);
@@ -925,15 +926,8 @@ int hse_plan_create(hse_plan* out, const hse_problem* p) {
       plan->split_buf_elems = buf;
     }
     HSE_TRY(plan_malloc(plan, &plan->comp_buf, comp * sizeof(float2)));
-    if (plan->apply_variant == kTwoVariant && plan->blocked) {
-      // the blocked copies of every pass, so that no call of the plan allocates or moves them: the
-      // first apply can be captured into a graph, and a later pass leaves that graph's copies in place
-      const size_t own = (size_t)nk * p->n_tgt, occ = (size_t)nkq * p->n_occ;
-      plan->blk_elems = std::max(2 * own + occ, (size_t)nk * p->n_occ + occ) * blocked_stride(n1);
-      HSE_TRY(plan_malloc(plan, &plan->blk_buf, plan->blk_elems * sizeof(float2)));
-    }
   }
-  size_t e64_items = 0;
+  size_t e64_items = 0, split64_bytes = 0;
   if (plan->p.dtype == HSE_C128 && f64_grid_bytes(n1, n2, n3) <= kF64MaxSmem) {
     int sms = 0;
     HSE_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, plan->device));
@@ -943,7 +937,6 @@ int hse_plan_create(hse_plan* out, const hse_problem* p) {
     const long long partners[3] = {(long long)nkq * p->n_occ,
                                    plan->sampled ? (long long)nkq * p->n_occ : (long long)nk * p->n_occ / 2 + 1,
                                    (long long)nk * p->n_tgt};
-    size_t buf = 0;
     for (int o = 0; o < 3; ++o) {
       const size_t out_bytes = o == ROLE_ENERGY ? 0 : (size_t)k_own[o] * owners[o] * N * sizeof(double2);
       SplitChoice best;
@@ -972,9 +965,8 @@ int hse_plan_create(hse_plan* out, const hse_problem* p) {
       if (log_on())
         std::fprintf(stderr, "hse: FP64 role %d: fused with %d orbitals a CTA and %d ranges %.0f us, staged %.0f us (estimates)\n",
                      o, plan->f64_T[o], best.ns, best.seconds * 1e6, staged * 1e6);
-      if (plan->fused64[o] && best.ns > 1) buf = std::max(buf, best.ns * out_bytes);
+      if (plan->fused64[o] && best.ns > 1) split64_bytes = std::max(split64_bytes, best.ns * out_bytes);
     }
-    if (buf) HSE_TRY(plan_malloc(plan, &plan->split64, buf));
     if (plan->fused64[ROLE_ENERGY])
       e64_items = (size_t)plan->f64_ns[ROLE_ENERGY] * (((size_t)nk * p->n_occ + plan->f64_T[ROLE_ENERGY] - 1) / plan->f64_T[ROLE_ENERGY]);
   }
@@ -1013,6 +1005,31 @@ int hse_plan_create(hse_plan* out, const hse_problem* p) {
       HSE_TRY(plan_malloc(plan, &plan->work, plan->work_pairs * N * sizeof(double2)));
     HSE_TRY(plan_malloc(plan, &plan->vx64, (size_t)nk * nown * N * sizeof(double2)));
   }
+  // what the plan can do without: where there is no memory for it, one range of partners, or the
+  // staged kernel
+  if (split64_bytes) {
+    e = plan_malloc(plan, &plan->split64, split64_bytes);
+    if (e == cudaErrorMemoryAllocation) {
+      cudaGetLastError();
+      plan->f64_ns[ROLE_TGT] = plan->f64_ns[ROLE_OCC] = 1;
+    } else {
+      HSE_TRY(e);
+    }
+  }
+  if (plan->apply_variant == kTwoVariant && plan->blocked && lone) {
+    // the blocked copies of every pass, so that no call of the plan allocates or moves them: the
+    // first apply can be captured into a graph, and a later pass leaves that graph's copies in place
+    const size_t own = (size_t)nk * p->n_tgt, occ = (size_t)nkq * p->n_occ;
+    plan->blk_elems = std::max(2 * own + occ, (size_t)nk * p->n_occ + occ) * blocked_stride(n1);
+    e = plan_malloc(plan, &plan->blk_buf, plan->blk_elems * sizeof(float2));
+    if (e == cudaErrorMemoryAllocation) {
+      cudaGetLastError();
+      plan->blk_elems = 0;
+      plan->apply_variant = 0;
+    } else {
+      HSE_TRY(e);
+    }
+  }
   TableArgs t{};
   t.qvec = plan->qvec;
   t.nq = plan->nq;
@@ -1048,6 +1065,11 @@ int hse_plan_create(hse_plan* out, const hse_problem* p) {
   }
   *out = plan;
   return HSE_OK;
+}
+
+int hse_plan_create(hse_plan* out, const hse_problem* p) {
+  const NvtxRange nvtx_range("hse_plan_create");
+  return create_plan(out, p, true);
 }
 
 int hse_status(hse_plan plan, hse_stream_t stream) {
@@ -1138,13 +1160,20 @@ int kernel_variant(hse_plan plan, int mode) {
 
 int run_pairconv(hse_plan plan, int mode, PairArgs a, int n_own, cudaStream_t st) {
   const int n = plan->p.grid[0];
-  const int variant = kernel_variant(plan, mode);
-  const int T = owner_slots(n, variant);
+  int variant = kernel_variant(plan, mode);
   a.n_own = n_own;
   if (variant != kWideVariant && pairconv_c64_pencil_load(n, mode, variant) && plan->blocked) {
     const int rc = to_blocked(plan, mode, a, st);
-    if (rc) return rc;
+    if (rc == HSE_ERR_NOMEM && mode == MODE_APPLY && variant == kTwoVariant) {
+      // the staged kernel needs no copies (and has the same tiles); the plan keeps to it
+      cudaGetLastError();
+      plan->apply_variant = 0;
+      variant = plan->blocks_per_sm;
+    } else if (rc) {
+      return rc;
+    }
   }
+  const int T = owner_slots(n, variant);
   a.ntiles = (n_own + T - 1) / T;
   a.nsplit = plan->nsplit[role_of(mode)];
   const size_t count = (size_t)a.nk_own * n_own * plan->N;
@@ -1870,7 +1899,7 @@ int hse_plan_create_batched(hse_plan* out, const hse_problem* cells, int ncells)
   size_t max_items = 0;
   for (int c = 0; c < ncells && rc == HSE_OK && e == cudaSuccess; ++c) {
     hse_plan sub = nullptr;
-    rc = hse_plan_create(&sub, &cells[c]);
+    rc = create_plan(&sub, &cells[c], false);
     if (rc) break;
     plan->cells.push_back(sub);
     const hse_problem& q = sub->p;
