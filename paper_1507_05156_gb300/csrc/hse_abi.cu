@@ -531,7 +531,7 @@ F64Rate f64_rate(int n1, int n2, int n3, int T) {
   return r;
 }
 constexpr double kWidePairSeconds = 7.1e-6;  // one partner of a tile of the two-exchange 16^3 kernel,
-constexpr double kWideOccSeconds = 17e-6;  // of its u_occ pass (two chains; 14.7 without omega, 18 with),
+constexpr double kWideOccSeconds = 17e-6;  // of its u_occ pass (two chains; 14.7 without omega, 18.6 with),
 constexpr double kPencilOccSeconds16 = 9.4e-6;  // and of the pencil-load kernel's u_occ pass (a two-owner tile)
 
 // Number of ranges the partners (k', j) of an owner tile are split into: the smallest estimated

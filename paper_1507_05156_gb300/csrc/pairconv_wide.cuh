@@ -538,9 +538,9 @@ __global__ void __launch_bounds__(Wide16::THREADS, 1)
 // spectrum A and the second adds Re sum_G dv A conj(B), as stage_x_occ does.  A takes the owner's
 // TMEM columns and the owner comes from a copy in the order of the threads (args.spec, one blocked
 // grid a slot), which 32 loads fetch at the start of a chain, when the registers are free for all of
-// them.  Of the 250 us omega costs, those loads are 136, the loads of dv 50 (A in that scratch and the
-// owner in TMEM: 290 us, its loads a few at a time between live spectra).
-// 16^3, 3^3 k, 8 bands: 1,440 us on the pencil-load kernel with omega, 1,383 here; 1,333 and 1,133 us
+// them.  Of the 299 us omega costs, those loads are 136, the loads of dv 50, the FP64 sums of 16 products each 46
+// (A in that scratch and the owner in TMEM: 40 more, its loads a few at a time between live spectra).
+// 16^3, 3^3 k, 8 bands: 1,546 us on the pencil-load kernel with omega, 1,429 here; 1,387 and 1,130 us
 // without.
 template <bool FUSE_W>
 __global__ void __launch_bounds__(Wide16::THREADS, 1)
@@ -687,9 +687,9 @@ __global__ void __launch_bounds__(Wide16::THREADS, 1)
               for (int k2 = 0; k2 < 4; ++k2) tmem_put_row32(town + (uint32_t)(32 * k2), reinterpret_cast<const float*>(v[k2]));
               tmem_wait_st();
             } else if (FUSE_W) {
-              float d = 0.f;
 #pragma unroll
               for (int k2 = 0; k2 < 4; ++k2) {
+                float d = 0.f;
                 float2 a[16];
                 tmem_issue_row32(town + (uint32_t)(32 * k2), reinterpret_cast<float*>(a));
                 float w[16];
@@ -701,8 +701,8 @@ __global__ void __launch_bounds__(Wide16::THREADS, 1)
                   const int i = wide_slot(y);
                   d = fmaf(w[y], fmaf(a[i].x, v[k2][i].x, a[i].y * v[k2][i].y), d);
                 }
+                wsum += (double)d;  // 16 products to an FP32 sum, as in the pencil kernels
               }
-              wsum += (double)d * (double)(args.scale * f);
             }
             wide_scale(v, row + t, f);
           },
@@ -721,7 +721,7 @@ __global__ void __launch_bounds__(Wide16::THREADS, 1)
   }
   if (active) wide_fold(tacc, sums, t, out, pl.hi, pl.lo, folds == 0, folds == 1, true);
   if constexpr (FUSE_W) {  // the item's share of d/d omega, one FP64 partial
-    red[tid] = active ? wsum : 0.0;
+    red[tid] = active ? wsum * (double)(args.scale * f) : 0.0;
     __syncthreads();
     if (tid == 0) {
       double sum = 0.0;
