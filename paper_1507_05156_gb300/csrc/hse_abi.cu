@@ -540,13 +540,14 @@ constexpr double kPencilOccSeconds16 = 9.4e-6;  // and of the pencil-load kernel
 // the pass that sums the ranges' outputs (4 us, 0.1 us a range and 3 TB/s over ns outputs).  A worker is a
 // resident CTA, or an SM that several CTAs share; its last item then runs alone, t_tail a pair
 // longer.  A finer split must gain 1%.  Beyond 48 waves the last one no longer matters.
+constexpr int kMaxRanges = 32;
 struct SplitChoice {
   int ns = 1;
   double seconds = 0.0;
 };
 SplitChoice choose_split(long long tiles, long long partners, double t_pair, long long slots, size_t out_bytes,
                          int ns_min, double t_item = 4e-6, double t_tail = 0.0) {
-  const int ns_cap = (int)std::min<long long>(32, partners);
+  const int ns_cap = (int)std::min<long long>(kMaxRanges, partners);
   const long long most = 48 * slots;
   SplitChoice best;
   best.ns = std::min(ns_min, ns_cap);
@@ -632,6 +633,13 @@ void* ortho_block(hse_plan plan, int nbands, cudaStream_t st) {
   }
   plan->ortho_blocks.push_back(b);
   return b.p;
+}
+
+// Test hooks of the launch shape, read when a plan is created (0: off): HSE_RANGES, the number of
+// partner ranges of every pass, and HSE_F64_TILE, the orbitals a CTA of the fused FP64 passes.
+int shape_from_env(const char* name, long long most) {
+  const char* env = std::getenv(name);
+  return env ? (int)std::clamp<long long>(std::atoll(env), 0, most) : 0;
 }
 
 bool invert3(const double* A, double* inv) {
@@ -912,6 +920,7 @@ static int create_plan(hse_plan* out, const hse_problem* p, bool lone) {
         consider(plan->occ_variant, kWideVariant, kWideSlots, kWideOccSeconds, sms, 0.0);
       }
       int best = choice.ns;
+      if (const int v = shape_from_env("HSE_RANGES", std::min<long long>(kMaxRanges, partners))) best = v;
       size_t need = (best > 1 && o != ROLE_ENERGY) ? (size_t)best * k_own[o] * owners[o] * N : 0;
       if (need * sizeof(float2) > ((size_t)4 << 30)) {  // keep split buffers modest
         best = 1;
@@ -955,6 +964,9 @@ static int create_plan(hse_plan* out, const hse_problem* p, bool lone) {
           plan->f64_T[o] = T;
         }
       }
+      const int most_T = (int)std::min<size_t>(16, kF64MaxSmem / f64_grid_bytes(n1, n2, n3));
+      if (const int v = shape_from_env("HSE_F64_TILE", most_T)) plan->f64_T[o] = v;
+      if (const int v = shape_from_env("HSE_RANGES", std::min<long long>(kMaxRanges, partners[o]))) best.ns = v;
       // the staged form: nine launches a target k-point, 0.84 TFLOP/s once they are full (0.93 at 24^3)
       const double pairs = (double)nk * owners[o] * nkq * p->n_occ * (o == ROLE_OCC ? 2.0 * p->n_tgt / p->n_occ : 1.0);
       const double Nd = (double)N;
