@@ -289,7 +289,7 @@ __device__ __forceinline__ bool staged_item(const PairArgs& args, const CUtensor
   const float2* lhs = (MODE == MODE_DOT) ? args.part2 + ((size_t)k * args.n_own + bandc) * G::N : own;
   double dsum = 0.0;
   int folds = 0;
-  const int fspan = fold_span(args.n_part);
+  const int fspan = fold_span(args.n_part, args.nk_part);
   auto fold = [&](bool last) {
 #pragma unroll 1
     for (int ps = 0; ps < (reg ? Lay::PPT : 0); ++ps) {

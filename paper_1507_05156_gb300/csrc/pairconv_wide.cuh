@@ -460,7 +460,7 @@ __global__ void __launch_bounds__(Wide16::THREADS, 1)
   float2* ga = g + wide_a(pl.hi, pl.lo, 0, 0);
   float2* gb = g + wide_b(pl.hi, pl.lo, 0, 0);
   const int p0 = pl.hi * 16 + pl.lo;  // staged row of r = 0
-  const int fspan = fold_span(args.n_part);
+  const int fspan = fold_span(args.n_part, args.nk_part);
   int folds = 0;
   uint32_t phases = 0;  // bit b: parity that stage buffer b completes next
   int buf = 0, cur_kp = -1;
@@ -618,7 +618,7 @@ __global__ void __launch_bounds__(Wide16::THREADS, 1)
   const int p0 = pl.hi * 16 + pl.lo;
   const float f = active ? (float)args.occ[it.k * args.n_occ + band] : 0.f;
   double wsum = 0.0;
-  const int fspan = fold_span(args.n_part);
+  const int fspan = fold_span(args.n_part, args.nk_part);
   int folds = 0, cur_kp = -1;
   const float* dv0 = nullptr;
   for (int q = 0; q < npairs; ++q) {
