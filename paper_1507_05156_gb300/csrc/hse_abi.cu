@@ -284,10 +284,10 @@ __global__ void scatter_rows(uint64_t* __restrict__ dst, const uint64_t* __restr
 
 using namespace hse;
 
-// Roles of the fused kernel's owners, each with its own k' split: targets (apply, VJP
-// w.r.t. u_tgt and omega), occupied orbitals at every target k-point (exchange energy),
-// occupied orbitals at the sampled k' (VJP w.r.t. u_occ).
-enum OwnerRole : int { ROLE_TGT = 0, ROLE_ENERGY = 1, ROLE_OCC = 2 };
+// Roles of the fused kernel's owners, each with its own ranges of partners: targets (apply, VJP
+// w.r.t. u_tgt), occupied orbitals at every target k-point (exchange energy), occupied
+// orbitals at the sampled k' (VJP w.r.t. u_occ), targets of the omega gradient alone.
+enum OwnerRole : int { ROLE_TGT = 0, ROLE_ENERGY = 1, ROLE_OCC = 2, ROLE_DOT = 3 };
 
 // Streams (branches of the captured graph) of the per-cell batched form: each cell's
 // single-cell launches go to the branch with the least work so far, so that a cell's last
@@ -328,7 +328,7 @@ struct hse_plan_s {
   int inject = 0;            // test hook (HSE_INJECT_SKIP_FILL=1 at plan creation)
   long long alloc_count = 0;   // device allocations made by this plan so far (plan_malloc)
   long long fail_alloc_at = -1;  // test hook (HSE_FAIL_ALLOC_AT=k at plan creation): allocation k fails
-  int nsplit[3] = {1, 1, 1};  // k'-loop splits of the fused kernel per OwnerRole
+  int nsplit[4] = {1, 1, 1, 1};  // k'-loop splits of the fused kernel per OwnerRole
   float2* split_buf = nullptr;  // [nsplit][nk_own][n_own][N] partial outputs when nsplit > 1
   size_t split_buf_elems = 0;
   float2* comp_buf = nullptr;   // [nsplit][nk_own][n_own][2][blocked] running sums s, c (APPLY / OCC)
@@ -493,19 +493,45 @@ struct BatchShape {
 
 int side_slot(int n) { return n == 8 ? 0 : n == 16 ? 1 : n == 18 ? 2 : n == 20 ? 3 : n == 12 ? 4 : -1; }
 
-// Seconds one SM spends on a pair convolution of grid side n: 41 TFLOP/s of 10 N log2 N + 16 N
-// flops on 152 SMs (16^3 and 24^3; only the ratio to the fixed costs below matters).
-double pair_seconds(int n) {
-  const double N = (double)n * n * n;
-  return (10.0 * N * std::log2(N) + 16.0 * N) / 0.27e12;
+// Seconds a work item takes: `item` for its start, its owners and its result, `pair` for a partner of its
+// tile (with a share of the kernel rows and folds), `tail` more for a partner while it has an SM alone that
+// could hold another item beside it.  Measured on the kernels that the default variants run, items of 4 to 32
+// partners in one, two and four waves (all within 3% of such a fit): the owner = target passes one CTA an SM,
+// the u_occ pass the time of an SM that two CTAs share (24^3: one), its item between those without and with
+// the omega gradient.  The dot passes end in a sum by one thread an owner, hence their items.
+struct PassRate {
+  double pair, item, tail;
+};
+PassRate pass_rate(int n, int role) {
+  static constexpr double us[9][4][3] = {
+      // V_x u          energy            u_occ              omega alone
+      {{1.20, 2.5, 0}, {1.44, 3.2, 0}, {2.2, 2.5, 1.1}, {1.20, 7.0, 0}},    // 4^3
+      {{1.78, 3.6, 0}, {2.07, 4.5, 0}, {4.3, 3.5, 0.7}, {1.78, 9.8, 0}},    // 6^3
+      {{1.99, 3.6, 0}, {2.10, 6.1, 0}, {4.0, 4.8, 1.1}, {1.99, 8.5, 0}},    // 8^3
+      {{2.59, 4.3, 0}, {2.59, 7.5, 0}, {4.9, 6.0, 1.1}, {2.59, 8.1, 0}},    // 10^3
+      {{3.67, 5.4, 0}, {3.67, 10.3, 0}, {7.5, 7.5, 1.2}, {3.67, 11.0, 0}},  // 12^3
+      {{4.20, 7.3, 0}, {4.00, 14.4, 0}, {9.4, 5.5, 1.4}, {4.00, 15.9, 0}},  // 16^3
+      {{3.77, 5.2, 0}, {3.77, 15.3, 0}, {7.9, 6.5, 2.8}, {3.77, 16.2, 0}},  // 18^3
+      {{4.84, 8.8, 0}, {4.84, 20.9, 0}, {10.3, 10.5, 2.5}, {4.84, 24.1, 0}}, // 20^3
+      {{7.40, 5.0, 0}, {7.20, 31.6, 0}, {17.8, 8.0, 0} , {7.40, 40.2, 0}},   // 24^3
+  };
+  const int side = n <= 12 ? n / 2 - 2 : n <= 16 ? 5 : n <= 18 ? 6 : n <= 20 ? 7 : 8;
+  const double* r = us[side][role];
+  return {r[0] * 1e-6, r[1] * 1e-6, r[2] * 1e-6};
 }
-// A partner of an owner tile on an SM: the staged kernel and the two-CTA kernel.
-double staged_seconds(int n) {
-  return n == 8 ? 2.06e-6 : n == 10 ? 2.64e-6 : n == 12 ? 3.85e-6 : n == 18 ? 3.86e-6 : 4.93e-6;
+// The same of the two-CTA kernel, of an SM that two CTAs share.
+PassRate two_cta_rate(int n) {
+  switch (n) {
+    case 8: return {1.78e-6, 0.9e-6, 0.5e-6};
+    case 10: return {2.00e-6, 1.0e-6, 0.5e-6};
+    case 12: return {3.27e-6, 1.6e-6, 0.9e-6};
+    case 18: return {3.24e-6, 1.5e-6, 0.9e-6};
+    default: return {4.16e-6, 2.3e-6, 1.2e-6};
+  }
 }
-double two_cta_seconds(int n) {
-  return n == 8 ? 1.91e-6 : n == 10 ? 2.15e-6 : n == 12 ? 3.52e-6 : n == 18 ? 3.48e-6 : 4.47e-6;
-}
+// The two-exchange kernels of 16^3, for a partner of four owners: the apply, and the u_occ pass (14.7 us
+// without omega, 18.6 with).
+constexpr PassRate kWideRate = {7.1e-6, 14e-6, 0.0}, kWideOccRate = {15.5e-6, 8e-6, 0.0};
 
 // The fused FP64 kernel with T orbitals a CTA: CTAs an SM holds, seconds of an SM a partner takes
 // when they are all busy (6.5 GFLOP/s of the same count; a partial warp costs a whole one, and with
@@ -530,23 +556,24 @@ F64Rate f64_rate(int n1, int n2, int n3, int T) {
   r.t_pipe = std::max(r.t_pipe, r.t_alone / r.ctas);
   return r;
 }
-constexpr double kWidePairSeconds = 7.1e-6;  // one partner of a tile of the two-exchange 16^3 kernel,
-constexpr double kWideOccSeconds = 17e-6;  // of its u_occ pass (two chains; 14.7 without omega, 18.6 with),
-constexpr double kPencilOccSeconds16 = 9.4e-6;  // and of the pencil-load kernel's u_occ pass (a two-owner tile)
 
 // Number of ranges the partners (k', j) of an owner tile are split into: the smallest estimated
-// time of list-scheduling `tiles` x ns ranges (partners / ns pairs of t_pair seconds, uneven where
-// ns does not divide, and t_item an item for its start, owner and result) on `slots` workers, plus
-// the pass that sums the ranges' outputs (4 us, 0.1 us a range and 3 TB/s over ns outputs).  A worker is a
-// resident CTA, or an SM that several CTAs share; its last item then runs alone, t_tail a pair
-// longer.  A finer split must gain 1%.  Beyond 48 waves the last one no longer matters.
+// time of list-scheduling `tiles` x ns ranges (partners / ns pairs, uneven where ns does not divide,
+// and an item's own time) on `slots` workers, plus the pass that sums the ranges' outputs, where there are
+// any (4 us, 0.1 us a range and 3 TB/s over ns outputs).  A worker is a
+// resident CTA, or an SM that several CTAs share; its last item then runs alone, `tail` a pair
+// longer.  A finer split must gain 1%.  Beyond 48 waves the last one no longer matters.  `host`: what the
+// host takes for the call and for one more launch, which a call's GPU time hides only if it is longer.
 constexpr int kMaxRanges = 32;
 struct SplitChoice {
   int ns = 1;
   double seconds = 0.0;
 };
-SplitChoice choose_split(long long tiles, long long partners, double t_pair, long long slots, size_t out_bytes,
-                         int ns_min, double t_item = 4e-6, double t_tail = 0.0) {
+struct HostTime {
+  double call = 0.0, launch = 0.0;
+};
+SplitChoice choose_split(long long tiles, long long partners, const PassRate& r, long long slots, size_t out_bytes,
+                         int ns_min, double t_sum = 4e-6, HostTime host = {}) {
   const int ns_cap = (int)std::min<long long>(kMaxRanges, partners);
   const long long most = 48 * slots;
   SplitChoice best;
@@ -555,11 +582,11 @@ SplitChoice choose_split(long long tiles, long long partners, double t_pair, lon
     if (best.seconds > 0.0 && (tiles * ns > most || (size_t)ns * out_bytes > ((size_t)4 << 30))) break;
     double t = 0.0;
     if (tiles * ns > most) {
-      t = (double)tiles * ((double)partners * t_pair + ns * t_item) / (double)slots;
+      t = (double)tiles * ((double)partners * r.pair + ns * r.item) / (double)slots;
     } else {
       std::map<double, long long> ends{{0.0, slots}};  // end time -> slots that end then
       for (int sp = 0; sp < ns; ++sp) {
-        const double cost = (double)((sp + 1) * partners / ns - sp * partners / ns) * t_pair + t_item;
+        const double cost = (double)((sp + 1) * partners / ns - sp * partners / ns) * r.pair + r.item;
         for (long long left = tiles; left > 0;) {  // the items of a range cost the same
           const auto first = ends.begin();
           const double end = first->first + cost;
@@ -571,8 +598,9 @@ SplitChoice choose_split(long long tiles, long long partners, double t_pair, lon
         }
       }
     }
-    t += t_tail * (double)((partners + ns - 1) / ns);
-    if (ns > 1) t += 4e-6 + ns * (0.1e-6 + (double)out_bytes / 3e12);
+    t += r.tail * (double)((partners + ns - 1) / ns);
+    if (ns > 1 && t_sum > 0.0) t += t_sum + ns * (0.1e-6 + (double)out_bytes / 3e12);
+    t = std::max(t, host.call + (ns > 1 ? host.launch : 0.0));
     if (best.seconds == 0.0 || t < 0.99 * best.seconds) {
       best.seconds = t;
       best.ns = ns;
@@ -883,12 +911,12 @@ static int create_plan(hse_plan* out, const hse_problem* p, bool lone) {
     const int occ_blocks = std::max(1, pairconv_c64_occupancy(n1, MODE_APPLY, plan->blocks_per_sm));
     const long long slots = (long long)sms * occ_blocks;
     // per OwnerRole: owner bands, owner k-points, partner k-points, partner bands
-    const int owners[3] = {p->n_tgt, p->n_occ, p->n_occ};
-    const int k_own[3] = {nk, nk, nkq};
-    const int k_part[3] = {nkq, nkq, nk};
-    const int b_part[3] = {p->n_occ, p->n_occ, p->n_tgt};
+    const int owners[4] = {p->n_tgt, p->n_occ, p->n_occ, p->n_tgt};
+    const int k_own[4] = {nk, nk, nkq, nk};
+    const int k_part[4] = {nkq, nkq, nk, nkq};
+    const int b_part[4] = {p->n_occ, p->n_occ, p->n_tgt, p->n_occ};
     size_t buf = 0, comp = 0;
-    for (int o = 0; o < 3; ++o) {
+    for (int o = 0; o < 4; ++o) {
       const int T = slots_for(n1);
       const long long partners = (long long)k_part[o] * b_part[o];
       // the staged-partner kernel (roles with owner = target) caches an item's occupations:
@@ -896,39 +924,42 @@ static int create_plan(hse_plan* out, const hse_problem* p, bool lone) {
       const int ns_min = (plan->blocks_per_sm <= 0 && o != ROLE_OCC)
                              ? (int)std::min<long long>(8, (partners + kOccCache - 1) / kOccCache)
                              : 1;
-      const double t_pair = (o == ROLE_OCC ? 2.0 : 1.0) * T * pair_seconds(n1);
-      const size_t out_bytes = o == ROLE_ENERGY ? 0 : (size_t)k_own[o] * owners[o] * N * sizeof(float2);
+      const bool outputs = o == ROLE_TGT || o == ROLE_OCC;  // else a double an owner and range
+      const size_t out_bytes = outputs ? (size_t)k_own[o] * owners[o] * N * sizeof(float2) : 0;
+      // a call with nothing but the kernel takes the host about 12 us, another launch 3
+      const HostTime host = o == ROLE_TGT ? HostTime{12e-6, 3e-6} : HostTime{};
       auto tiles = [&](int per) { return (long long)k_own[o] * ((owners[o] + per - 1) / per); };
-      SplitChoice choice = choose_split(tiles(T), partners, t_pair, slots, out_bytes, ns_min);
+      auto choose = [&](int per, const PassRate& r, long long workers) {
+        return choose_split(tiles(per), partners, r, workers, out_bytes, ns_min, outputs ? 4e-6 : 0.0, host);
+      };
+      SplitChoice choice = choose(T, pass_rate(n1, o), o == ROLE_OCC ? sms : slots);
       // another kernel of the pass takes it where its estimate is shorter
-      auto consider = [&](int& chosen, int variant, int per, double t_other, long long workers, double extra) {
-        SplitChoice c = choose_split(tiles(per), partners, t_other, workers, out_bytes, ns_min);
+      auto consider = [&](int& chosen, int variant, int per, const PassRate& r, long long workers, double extra) {
+        SplitChoice c = choose(per, r, workers);
         c.seconds += extra;
         if (chosen == 0 && c.seconds < choice.seconds) chosen = variant;
         if (chosen == variant) choice = c;
       };
       if (plan->blocks_per_sm == 0 && o == ROLE_TGT && n1 == 16)
-        consider(plan->apply_variant, kWideVariant, kWideSlots, kWidePairSeconds, sms, 0.0);
-      if (plan->blocks_per_sm == 0 && o == ROLE_TGT && two_cta_fits(n1)) {
-        // two CTAs share an SM; the pencil-blocked copies cost two launches and three passes
-        const double copies = 8e-6 + 3.0 * N * sizeof(float2) * ((double)nk * p->n_tgt + (double)nkq * p->n_occ) / 4e12;
-        choice = choose_split(tiles(T), partners, staged_seconds(n1), slots, out_bytes, ns_min);
-        consider(plan->apply_variant, kTwoVariant, T, 2.0 * two_cta_seconds(n1), 2 * sms, copies);
-      }
-      if (plan->blocks_per_sm == 0 && o == ROLE_OCC && n1 == 16) {
-        choice = choose_split(tiles(T), partners, kPencilOccSeconds16, slots, out_bytes, ns_min);
-        consider(plan->occ_variant, kWideVariant, kWideSlots, kWideOccSeconds, sms, 0.0);
-      }
+        consider(plan->apply_variant, kWideVariant, kWideSlots, kWideRate, sms, 0.0);
+      // the pencil-blocked copies cost a launch and a few passes each: two arrays here, three in the u_occ pass
+      auto copies = [&](int arrays, double orbitals) { return arrays * 4e-6 + 3.0 * N * sizeof(float2) * orbitals / 4e12; };
+      if (plan->blocks_per_sm == 0 && o == ROLE_TGT && two_cta_fits(n1))
+        consider(plan->apply_variant, kTwoVariant, T, two_cta_rate(n1), sms,
+                 copies(2, (double)nk * p->n_tgt + (double)nkq * p->n_occ));
+      if (plan->blocks_per_sm == 0 && o == ROLE_OCC && n1 == 16)  // makes none
+        consider(plan->occ_variant, kWideVariant, kWideSlots, kWideOccRate, sms,
+                 -copies(3, 2.0 * nk * p->n_tgt + (double)nkq * p->n_occ));
       int best = choice.ns;
       if (const int v = shape_from_env("HSE_RANGES", std::min<long long>(kMaxRanges, partners))) best = v;
-      size_t need = (best > 1 && o != ROLE_ENERGY) ? (size_t)best * k_own[o] * owners[o] * N : 0;
+      size_t need = (best > 1 && outputs) ? (size_t)best * k_own[o] * owners[o] * N : 0;
       if (need * sizeof(float2) > ((size_t)4 << 30)) {  // keep split buffers modest
         best = 1;
         need = 0;
       }
       plan->nsplit[o] = best;
       if (best > 1) buf = std::max(buf, need);
-      if (o != ROLE_ENERGY) comp = std::max(comp, (size_t)best * k_own[o] * owners[o] * 2 * blocked_stride(n1));
+      if (outputs) comp = std::max(comp, (size_t)best * k_own[o] * owners[o] * 2 * blocked_stride(n1));
     }
     if (buf) {
       HSE_TRY(plan_malloc(plan, &plan->split_buf, buf * sizeof(float2)));
@@ -957,8 +988,8 @@ static int create_plan(hse_plan* out, const hse_problem* p, bool lone) {
                                                  : (long long)k_own[o] * ((owners[o] + T - 1) / T);
         const double pass = o == ROLE_ENERGY ? 0.45 : o == ROLE_OCC ? 2.0 : 1.0;
         const double t_pair = r.ctas > 1 ? r.t_pipe : r.t_alone;
-        const SplitChoice c = choose_split(tiles, partners[o], pass * t_pair, sms, out_bytes, 1, 1.5e-6 / r.ctas,
-                                           pass * (r.t_alone - t_pair));
+        const SplitChoice c = choose_split(tiles, partners[o], {pass * t_pair, 1.5e-6 / r.ctas, pass * (r.t_alone - t_pair)}, sms,
+                                           out_bytes, 1);
         if (T == 1 || c.seconds < 0.99 * best.seconds) {
           best = c;
           plan->f64_T[o] = T;
@@ -983,7 +1014,7 @@ static int create_plan(hse_plan* out, const hse_problem* p, bool lone) {
       e64_items = (size_t)plan->f64_ns[ROLE_ENERGY] * (((size_t)nk * p->n_occ + plan->f64_T[ROLE_ENERGY] - 1) / plan->f64_T[ROLE_ENERGY]);
   }
   {
-    const size_t np = std::max({(size_t)plan->nsplit[ROLE_TGT] * nk * p->n_tgt,
+    const size_t np = std::max({(size_t)plan->nsplit[ROLE_DOT] * nk * p->n_tgt,
                                 (size_t)plan->nsplit[ROLE_ENERGY] * nk * p->n_occ, e64_items});
     HSE_TRY(plan_malloc(plan, &plan->partial, std::max(np, (size_t)nk * nown) * sizeof(double)));
   }
@@ -1118,7 +1149,9 @@ PairArgs base_args(hse_plan plan) {
   return a;
 }
 
-int role_of(int mode) { return mode == MODE_ENERGY ? ROLE_ENERGY : (mode == MODE_OCC ? ROLE_OCC : ROLE_TGT); }
+int role_of(int mode) {
+  return mode == MODE_ENERGY ? ROLE_ENERGY : mode == MODE_OCC ? ROLE_OCC : mode == MODE_DOT ? ROLE_DOT : ROLE_TGT;
+}
 
 // Blocked layouts of the orbital arrays a pencil-load launch reads (own, part and, for
 // MODE_DOT / MODE_OCC, part2), in the plan's scratch; an array given twice is copied once.
