@@ -98,8 +98,8 @@ __global__ void to_pencil_blocks(float4* __restrict__ dst, const float4* __restr
 }
 
 // out[i] = sum_s buf[s * count + i], splits in ascending order (deterministic), compensated
-// (TwoSum, as the k' groups inside a split); eight loads in flight, which is what counts where the
-// outputs are few (8^3, 8 k, 4 bands, 16 splits: the apply 22.3 -> 20.7 us)
+// (TwoSum, as the k' groups inside a split); eight loads in flight (with one the sum of 16 splits at
+// 8^3, 8 k, 4 bands took 4.5 us; the whole call, 20 us, changes by less than its spread)
 __global__ void reduce_splits(float4* __restrict__ out, const float4* __restrict__ buf, int nsplit, size_t count4) {
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < count4; i += (size_t)gridDim.x * blockDim.x) {
     float4 a = buf[i], c = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -1153,6 +1153,17 @@ int role_of(int mode) {
   return mode == MODE_ENERGY ? ROLE_ENERGY : mode == MODE_OCC ? ROLE_OCC : mode == MODE_DOT ? ROLE_DOT : ROLE_TGT;
 }
 
+// Room for `need` elements of pencil-blocked copies.
+int grow_copies(hse_plan plan, size_t need) {
+  if (need <= plan->blk_elems) return HSE_OK;
+  cudaFree(plan->blk_buf);
+  plan->blk_buf = nullptr;
+  plan->blk_elems = 0;
+  const cudaError_t e = plan_malloc(plan, &plan->blk_buf, need * sizeof(float2));
+  if (e == cudaSuccess) plan->blk_elems = need;
+  return cuda_fail(e);
+}
+
 // Blocked layouts of the orbital arrays a pencil-load launch reads (own, part and, for
 // MODE_DOT / MODE_OCC, part2), in the plan's scratch; an array given twice is copied once.
 int to_blocked(hse_plan plan, int mode, PairArgs& a, cudaStream_t st) {
@@ -1167,14 +1178,8 @@ int to_blocked(hse_plan plan, int mode, PairArgs& a, cudaStream_t st) {
   if (mode == MODE_OCC) arrs[2].norb = (size_t)a.nk_part * a.n_part;
   size_t need = 0;
   for (const Arr& r : arrs) need += r.norb * nbk;
-  if (need > plan->blk_elems) {
-    cudaFree(plan->blk_buf);
-    plan->blk_buf = nullptr;
-    plan->blk_elems = 0;
-    const cudaError_t e = plan_malloc(plan, &plan->blk_buf, need * sizeof(float2));
-    if (e != cudaSuccess) return cuda_fail(e);
-    plan->blk_elems = need;
-  }
+  const int rc = grow_copies(plan, need);
+  if (rc) return rc;
   const float2* src[3] = {a.own, a.part, a.part2};
   const float2* dst[3] = {nullptr, nullptr, nullptr};
   size_t off = 0;
@@ -1203,20 +1208,34 @@ int kernel_variant(hse_plan plan, int mode) {
   return chosen ? chosen : plan->blocks_per_sm;
 }
 
+// Without memory for the copies of a two-CTA apply the plan keeps to the staged kernel, which needs none
+// (and has the same tiles).
+bool keep_to_staged(hse_plan plan, int rc, int variant) {
+  if (rc != HSE_ERR_NOMEM || variant != kTwoVariant) return false;
+  cudaGetLastError();
+  plan->apply_variant = 0;
+  return true;
+}
+
+// The copies of an apply, before the call that makes them: an autotuner's timing then has no allocation in it.
+int reserve_copies(hse_plan plan) {
+  const int variant = kernel_variant(plan, MODE_APPLY);
+  if (!plan->blocked || variant == kWideVariant || !pairconv_c64_pencil_load(plan->p.grid[0], MODE_APPLY, variant)) return HSE_OK;
+  const size_t orbitals = (size_t)plan->p.nk * plan->p.n_tgt + (size_t)plan->nkq * plan->p.n_occ;
+  const int rc = grow_copies(plan, orbitals * blocked_stride(plan->p.grid[0]));
+  return keep_to_staged(plan, rc, variant) ? HSE_OK : rc;
+}
+
 int run_pairconv(hse_plan plan, int mode, PairArgs a, int n_own, cudaStream_t st) {
   const int n = plan->p.grid[0];
   int variant = kernel_variant(plan, mode);
   a.n_own = n_own;
   if (variant != kWideVariant && pairconv_c64_pencil_load(n, mode, variant) && plan->blocked) {
     const int rc = to_blocked(plan, mode, a, st);
-    if (rc == HSE_ERR_NOMEM && mode == MODE_APPLY && variant == kTwoVariant) {
-      // the staged kernel needs no copies (and has the same tiles); the plan keeps to it
-      cudaGetLastError();
-      plan->apply_variant = 0;
+    if (keep_to_staged(plan, rc, variant))
       variant = plan->blocks_per_sm;
-    } else if (rc) {
+    else if (rc)
       return rc;
-    }
   }
   const int T = owner_slots(n, variant);
   a.ntiles = (n_own + T - 1) / T;
@@ -2105,6 +2124,10 @@ int hse_fock_apply_batched(hse_plan plan, const void* const* u_occ, const double
       if (e == cudaSuccess) e = cudaEventCreate(&t1);
       auto time_shape = [&](const BatchShape& s, float* ms) {
         apply(s);
+        for (hse_plan c : plan->cells) {
+          const int rc = s.percell ? reserve_copies(c) : HSE_OK;
+          if (rc != HSE_OK) return rc == HSE_ERR_NOMEM ? cudaErrorMemoryAllocation : cudaErrorUnknown;
+        }
         cudaError_t r = cudaMemcpyAsync(plan->d_cells, plan->h_cells.data(), ncells * sizeof(BatchCell),
                                         cudaMemcpyHostToDevice, st);
         if (r == cudaSuccess) r = cudaEventRecord(t0, st);
