@@ -164,7 +164,7 @@ struct ItemIdx {
 // ---------------------------------------------------------------------------------------
 // Compensated accumulation over k' (Sec. II C, Eq. "Fock": V_x u sums the pair terms over
 // every k' and every occupied band).  The TMEM accumulator of a pencil holds the sum over the
-// bands of a group of consecutive k' (in FP32; fold_span k-points).  When the group ends it is
+// bands of a group of consecutive k' (in FP32; at most fold_terms).  When the group ends it is
 // added to the pencil's running sum s with Knuth's TwoSum, whose exact rounding error is added to a second running sum c;
 // the pencil's result is s + c, written to the output (or the work item's split partial) by
 // the last fold.  s and c live in PairArgs::comp in the pencil-blocked layout (a warp's 32
@@ -173,12 +173,14 @@ struct ItemIdx {
 // an FP64 sum.
 // ---------------------------------------------------------------------------------------
 
-// k-points per fold group: one, or enough for 16 partner bands.  Over up to eight k-points of more than
-// eight bands always one: how finely a small problem's partners are split then does not lengthen the FP32
-// sums (24^3, 8 k, 13 bands, ranges of two k-points: errors of 1.26e-7 in sums of 26 terms, 1.10e-7 in 13,
-// for 2% more time; a fold costs about as much as a third of a pair).
-__host__ __device__ __forceinline__ int fold_span(int n_part, int nk_part) {
-  return n_part >= 16 || (n_part > 8 && nk_part <= 8) ? 1 : (16 + n_part - 1) / n_part;
+// Partner terms that a fold group may hold: a k' whose terms would take it past them starts another.  One
+// k-point's bands, or enough k-points for 16; over up to eight k-points no more than 16, so that how finely a
+// small problem's partners are split does not lengthen its FP32 sums (24^3, 8 k, 13 bands, ranges of two
+// k-points: errors of 1.26e-7 in sums of 26 terms, 1.10e-7 in 13, for 2% more time; a fold costs about as
+// much as a third of a pair).
+__host__ __device__ __forceinline__ int fold_terms(int n_part, int nk_part) {
+  if (n_part >= 16) return n_part;
+  return nk_part <= 8 ? 16 : (16 + n_part - 1) / n_part * n_part;
 }
 
 // a + b = s + err exactly, s = fl(a + b) (TwoSum; no fast-math reassociation in this build)
@@ -930,7 +932,8 @@ __device__ __forceinline__ void pairconv_item(const PairArgs& args, int item, fl
     }
   };
   if (it.q0 == it.q1) fold(true, false, true);  // no partners: zeros
-  const int fspan = fold_span(args.n_part, args.nk_part);
+  const int most = fold_terms(args.n_part, args.nk_part);
+  int folds = 0, group = 0;  // folds so far; terms of the current group
 
   // MODE_OCC with the omega gradient fused in: this slot's spectrum scratch and FP64 sum
   const bool fuse_w = MODE == MODE_OCC && args.vtab2 != nullptr && spec != nullptr;
@@ -981,9 +984,14 @@ __device__ __forceinline__ void pairconv_item(const PairArgs& args, int item, fl
         if (warp_on) stage_z_inverse<n, EPI_WCONJ, PPT, TS>(g, t, part, trow0, blk);
       }
     }
-    // the end of a fold group (fold_span k-points) or of the item's k' range
-    const int grp = (kp - kp_begin) / fspan;
-    if (kp == kp_end - 1 || (kp - kp_begin + 1) % fspan == 0) fold(grp == 0, grp == 1, kp == kp_end - 1);
+    // the end of the item, or of a fold group that the next k' would overfill
+    group += j1 - (kp == kp_begin ? j_begin : 0);
+    const bool last = kp == kp_end - 1;
+    if (last || group + (kp == kp_end - 2 ? j_end : args.n_part) > most) {
+      fold(folds == 0, folds == 1, last);
+      ++folds;
+      group = 0;
+    }
   }
 
   if constexpr (MODE == MODE_OCC) {

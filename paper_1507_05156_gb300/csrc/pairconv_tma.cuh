@@ -240,7 +240,7 @@ __device__ __forceinline__ bool staged_item(const PairArgs& args, const CUtensor
   const int band = it.tile * G::T + slot;
   const bool active = valid && band < args.n_own;
   const int bandc = active ? band : 0;
-  const int q0 = it.q0, npairs = it.q1 - it.q0, kp_begin = it.q0 / args.n_part;
+  const int q0 = it.q0, npairs = it.q1 - it.q0;
   const float2* own = args.own + ((size_t)k * args.n_own + bandc) * G::N;
 
   // fill stage buffer `buf` with partner q (warp 0 only)
@@ -289,7 +289,7 @@ __device__ __forceinline__ bool staged_item(const PairArgs& args, const CUtensor
   const float2* lhs = (MODE == MODE_DOT) ? args.part2 + ((size_t)k * args.n_own + bandc) * G::N : own;
   double dsum = 0.0;
   int folds = 0;
-  const int fspan = fold_span(args.n_part, args.nk_part);
+  const int most = fold_terms(args.n_part, args.nk_part);
   auto fold = [&](bool last) {
 #pragma unroll 1
     for (int ps = 0; ps < (reg ? Lay::PPT : 0); ++ps) {
@@ -331,13 +331,17 @@ __device__ __forceinline__ bool staged_item(const PairArgs& args, const CUtensor
   int buf = 0;
   int cur_kp = -1, kp_end = 0;  // the k' of the cached row, and the first partner past it (a division a pair
                                 // to tell costs 2 us in 54 at 4^3, 24 k, 8 + 8 bands)
+  int group_q = 0;              // first partner of the fold group
   while (q < npairs) {
     const float f = item_occ(sh.occ, args, q0, q);
     if (q >= kp_end) {
       const int kp = (q0 + q) / args.n_part;
       kp_end = (kp + 1) * args.n_part - q0;
-      // a new fold group (fold_span k-points) starts: fold the previous one
-      if (cur_kp >= 0 && (kp - kp_begin) / fspan != (cur_kp - kp_begin) / fspan) fold(false);
+      // a k' that would overfill the fold group starts another: fold the previous one
+      if (cur_kp >= 0 && min(kp_end, npairs) - group_q > most) {
+        fold(false);
+        group_q = q;
+      }
       const int qrow = args.qidx[k * args.nk_part + kp];
       if (on) Lay::cache_row(t, trow0, args.vtab + (size_t)qrow * G::N, args.scale);
       cur_kp = kp;
