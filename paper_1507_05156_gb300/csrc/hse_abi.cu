@@ -510,7 +510,7 @@ PassRate pass_rate(int n, int role) {
       {{1.99, 3.6, 0}, {2.10, 6.1, 0}, {4.0, 4.8, 1.1}, {1.99, 8.5, 0}},    // 8^3
       {{2.59, 4.3, 0}, {2.59, 7.5, 0}, {4.9, 6.0, 1.1}, {2.59, 8.1, 0}},    // 10^3
       {{3.67, 5.4, 0}, {3.67, 10.3, 0}, {7.5, 7.5, 1.2}, {3.67, 11.0, 0}},  // 12^3
-      {{4.20, 7.3, 0}, {4.00, 14.4, 0}, {9.4, 5.5, 1.4}, {4.00, 15.9, 0}},  // 16^3
+      {{4.20, 7.3, 0}, {4.00, 14.4, 0}, {8.8, 5.5, 1.4}, {4.00, 15.9, 0}},  // 16^3
       {{3.77, 5.2, 0}, {3.77, 15.3, 0}, {7.9, 6.5, 2.8}, {3.77, 16.2, 0}},  // 18^3
       {{4.84, 8.8, 0}, {4.84, 20.9, 0}, {10.3, 10.5, 2.5}, {4.84, 24.1, 0}}, // 20^3
       {{7.40, 5.0, 0}, {7.20, 31.6, 0}, {17.8, 8.0, 0} , {7.40, 40.2, 0}},   // 24^3
@@ -529,9 +529,9 @@ PassRate two_cta_rate(int n) {
     default: return {4.16e-6, 2.3e-6, 1.2e-6};
   }
 }
-// The two-exchange kernels of 16^3, for a partner of four owners: the apply, and the u_occ pass (14.7 us
-// without omega, 18.6 with).
-constexpr PassRate kWideRate = {7.1e-6, 14e-6, 0.0}, kWideOccRate = {15.5e-6, 8e-6, 0.0};
+// The two-exchange kernels of 16^3, for a partner of four owners: the apply, and the u_occ pass (14.9 us
+// without omega, 17.9 with, where two tiles of the pencil-load kernel's two owners take 17.0 and 18.9).
+constexpr PassRate kWideRate = {7.1e-6, 14e-6, 0.0}, kWideOccRate = {16.4e-6, 8e-6, 0.0};
 
 // The fused FP64 kernel with T orbitals a CTA: CTAs an SM holds, seconds of an SM a partner takes
 // when they are all busy (6.5 GFLOP/s of the same count; a partial warp costs a whole one, and with
@@ -563,17 +563,14 @@ F64Rate f64_rate(int n1, int n2, int n3, int T) {
 // any (4 us, 0.1 us a range and 3 TB/s over ns outputs).  A worker is a
 // resident CTA, or an SM that several CTAs share; its last item then runs alone, `tail` a pair
 // longer.  A finer split must gain 1%.  Beyond 48 waves the last one no longer matters.  `host`: what the
-// host takes for the call and for one more launch, which a call's GPU time hides only if it is longer.
+// host takes for a call with two launches; one range that is no longer is left whole.
 constexpr int kMaxRanges = 32;
 struct SplitChoice {
   int ns = 1;
   double seconds = 0.0;
 };
-struct HostTime {
-  double call = 0.0, launch = 0.0;
-};
 SplitChoice choose_split(long long tiles, long long partners, const PassRate& r, long long slots, size_t out_bytes,
-                         int ns_min, double t_sum = 4e-6, HostTime host = {}) {
+                         int ns_min, double t_sum = 4e-6, double host = 0.0) {
   const int ns_cap = (int)std::min<long long>(kMaxRanges, partners);
   const long long most = 48 * slots;
   SplitChoice best;
@@ -600,7 +597,7 @@ SplitChoice choose_split(long long tiles, long long partners, const PassRate& r,
     }
     t += r.tail * (double)((partners + ns - 1) / ns);
     if (ns > 1 && t_sum > 0.0) t += t_sum + ns * (0.1e-6 + (double)out_bytes / 3e12);
-    t = std::max(t, host.call + (ns > 1 ? host.launch : 0.0));
+    if (ns == 1 && t <= host) return {1, t};
     if (best.seconds == 0.0 || t < 0.99 * best.seconds) {
       best.seconds = t;
       best.ns = ns;
@@ -926,8 +923,7 @@ static int create_plan(hse_plan* out, const hse_problem* p, bool lone) {
                              : 1;
       const bool outputs = o == ROLE_TGT || o == ROLE_OCC;  // else a double an owner and range
       const size_t out_bytes = outputs ? (size_t)k_own[o] * owners[o] * N * sizeof(float2) : 0;
-      // a call with nothing but the kernel takes the host about 12 us, another launch 3
-      const HostTime host = o == ROLE_TGT ? HostTime{12e-6, 3e-6} : HostTime{};
+      const double host = o == ROLE_TGT ? 15e-6 : 0.0;  // 12 us a call, 3 the sum's launch
       auto tiles = [&](int per) { return (long long)k_own[o] * ((owners[o] + per - 1) / per); };
       auto choose = [&](int per, const PassRate& r, long long workers) {
         return choose_split(tiles(per), partners, r, workers, out_bytes, ns_min, outputs ? 4e-6 : 0.0, host);
