@@ -120,7 +120,9 @@ __global__ void __launch_bounds__(32 * kGramTiles, 2) gram_kernel(const C* __res
   const int k = blockIdx.y, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (skip && skip[k]) return;  // uniform over the cluster
   const int nt = (nb + 3) / 4, ntiles = nt * (nt + 1) / 2, P = 32 * R;
-  // 16 bands: diagonal tiles (0, 4, 7, 9; half the work) go to the schedulers that hold three warps
+  // 13 to 16 bands: diagonal tiles (0, 4, 7, 9; half the work) go to the schedulers that hold three warps
+  // of the ten.  More bands fill several groups of ten, of which only the last can be short; where a
+  // group's diagonal tiles lie differs from group to group, and its tiles keep their order.
   constexpr unsigned long long kOrder16 = 0x9786405321ull;
   const int wt = warp % tiles_here, rep = warp / tiles_here;
   const int tl = ntiles == 10 ? (int)((kOrder16 >> (4 * wt)) & 15) : wt;

@@ -423,7 +423,7 @@ __global__ void __launch_bounds__(Wide16::THREADS, 1)
   const int band = it.tile * W::SLOTS + slot;
   const bool active = band < args.n_own;  // uniform over the slot; an empty slot only passes the CTA barriers
   const int nwarps = 2 * min(W::SLOTS, args.n_own - it.tile * W::SLOTS);  // warps that use the stage
-  const int q0 = it.q0, npairs = it.q1 - it.q0;
+  const int q0 = it.q0, npairs = it.q1 - it.q0, kp_begin = it.q0 / args.n_part;
   for (int i = tid; i < npairs && i < kOccCache; i += W::THREADS) sh.occ[i] = partner_occ(args, q0 + i);
   tmem_fence_before_sync();
   __syncthreads();
@@ -460,8 +460,8 @@ __global__ void __launch_bounds__(Wide16::THREADS, 1)
   float2* ga = g + wide_a(pl.hi, pl.lo, 0, 0);
   float2* gb = g + wide_b(pl.hi, pl.lo, 0, 0);
   const int p0 = pl.hi * 16 + pl.lo;  // staged row of r = 0
-  const int most = fold_terms(args.n_part, args.nk_part);
-  int folds = 0, group_q = 0;  // folds so far; first partner of the fold group
+  const int fspan = fold_terms(args.n_part, args.nk_part) / args.n_part;
+  int folds = 0;
   uint32_t phases = 0;  // bit b: parity that stage buffer b completes next
   int buf = 0, cur_kp = -1;
   while (q < npairs) {
@@ -470,10 +470,9 @@ __global__ void __launch_bounds__(Wide16::THREADS, 1)
     if (kp != cur_kp) {  // uniform over the CTA
       float4 rv[4];
       wide_row_load(rv, args.vtab + (size_t)args.qidx[it.k * args.nk_part + kp] * W::N, args.scale);
-      if (cur_kp >= 0 && min((kp + 1) * args.n_part - q0, npairs) - group_q > most) {
-        if (active) wide_fold(tacc, sums, t, out, pl.hi, pl.lo, folds == 0, folds == 1, false);
+      if (active && cur_kp >= 0 && (kp - kp_begin) / fspan != (cur_kp - kp_begin) / fspan) {
+        wide_fold(tacc, sums, t, out, pl.hi, pl.lo, folds == 0, folds == 1, false);
         ++folds;
-        group_q = q;
       }
       __syncthreads();  // every slot is past its last use of the old row
       wide_row_store(rv, row);
@@ -577,7 +576,7 @@ __global__ void __launch_bounds__(Wide16::THREADS, 1)
   const int band = it.tile * W::SLOTS + slot;
   const bool active = band < args.n_own;  // uniform over the slot
   const int nwarps = 2 * min(W::SLOTS, args.n_own - it.tile * W::SLOTS);
-  const int npairs = it.q1 - it.q0;
+  const int npairs = it.q1 - it.q0, kp_begin = it.q0 / args.n_part;
   tmem_fence_before_sync();
   __syncthreads();
   tmem_fence_after_sync();
@@ -619,8 +618,8 @@ __global__ void __launch_bounds__(Wide16::THREADS, 1)
   const int p0 = pl.hi * 16 + pl.lo;
   const float f = active ? (float)args.occ[it.k * args.n_occ + band] : 0.f;
   double wsum = 0.0;
-  const int most = fold_terms(args.n_part, args.nk_part);
-  int folds = 0, group_q = 0, cur_kp = -1;
+  const int fspan = fold_terms(args.n_part, args.nk_part) / args.n_part;
+  int folds = 0, cur_kp = -1;
   const float* dv0 = nullptr;
   for (int q = 0; q < npairs; ++q) {
     const int kp = (it.q0 + q) / args.n_part;
@@ -628,10 +627,9 @@ __global__ void __launch_bounds__(Wide16::THREADS, 1)
       const size_t qrow = args.qidx[kp * args.nk_own + it.k];
       float4 rv[4];
       wide_row_load(rv, args.vtab + qrow * W::N, args.scale);
-      if (cur_kp >= 0 && min((kp + 1) * args.n_part - it.q0, npairs) - group_q > most) {
-        if (active) wide_fold(tacc, sums, t, out, pl.hi, pl.lo, folds == 0, folds == 1, false);
+      if (active && cur_kp >= 0 && (kp - kp_begin) / fspan != (cur_kp - kp_begin) / fspan) {
+        wide_fold(tacc, sums, t, out, pl.hi, pl.lo, folds == 0, folds == 1, false);
         ++folds;
-        group_q = q;
       }
       __syncthreads();  // every slot is past its last use of the old row
       wide_row_store(rv, row);
