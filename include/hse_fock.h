@@ -32,7 +32,10 @@
  * Calls are asynchronous on the caller's stream (a cudaStream_t passed as void*,
  * NULL = legacy default stream) and return an hse error code; device-side failures
  * are reported by hse_status.  The library never frees caller memory.  It allocates
- * only its plan (kernel tables and reduction scratch) in hse_plan_create*.
+ * only its plan (kernel tables and reduction scratch) in hse_plan_create*, and what the
+ * calls below say they allocate.  Calls on one plan share its scratch: order them, on one
+ * stream or by events (hse_overlap and complex128 hse_orthonormalize calls may overlap);
+ * calls on different plans are independent.
  */
 #ifndef HSE_FOCK_H
 #define HSE_FOCK_H
@@ -117,7 +120,8 @@ int hse_plan_destroy(hse_plan plan);
  * respect to u_occ at most sizes) copies the orbitals it reads into plan scratch in a
  * pencil-blocked layout, which the first such call (or one needing more than before)
  * allocates with device-wide synchronisation; plans whose apply runs that kernel at 8^3 to
- * 20^3 hold the copies from their creation. */
+ * 20^3 hold the copies from their creation (where there is no memory for them their apply runs
+ * the staged kernel). */
 int hse_fock_apply(hse_plan plan, const void *u_occ, const double *occ, const void *u_tgt,
                    void *vx_out, hse_stream_t stream);
 
@@ -274,7 +278,8 @@ int hse_overlap(hse_plan plan, const void *u, int nbands, double *S, hse_stream_
  * inner product and update in FP64.  Up to 64 bands that are well conditioned go through the
  * Cholesky factor of their overlap matrix (complex128: twice); the others, and a few small
  * bands, through modified Gram-Schmidt applied twice (complex64 ones in an FP64 copy).
- * complex64 bands are rounded once, when written back.  A band that is linearly dependent on the earlier ones (its norm after the
+ * complex64 bands are rounded once, when written back.  A band that is linearly dependent on
+ * the earlier ones (its norm after the
  * projections at most 1e-12 of its norm before them for complex128, 1e-5 for complex64, whose
  * rounding leaves about 1e-7 of any band outside the span of the others) is set to zero and
  * the plan's status word records HSE_ERR_SINGULAR (returned by hse_status).

@@ -423,8 +423,9 @@ def hse_overlap(plan: Plan, u: torch.Tensor, out: Optional[torch.Tensor] = None,
 
 
 def hse_orthonormalize(plan: Plan, u: torch.Tensor, stream=None) -> torch.Tensor:
-    """Orthonormalises u [nk][nb][grid] in place per k-point (FP64 modified Gram-Schmidt, twice);
-    a linearly dependent band surfaces as HSE_ERR_SINGULAR from hse_status."""
+    """Orthonormalises u [nk][nb][grid] in place per k-point, in band order and FP64 (by the Cholesky
+    factor of the overlaps where that is safe, else modified Gram-Schmidt twice); a linearly
+    dependent band surfaces as HSE_ERR_SINGULAR from hse_status."""
     lib = load_library()
     nb = _bands(plan, u)
     _check(lib.hse_orthonormalize(plan.handle, _ptr(u), nb, _stream(stream)), "hse_orthonormalize")

@@ -1,7 +1,7 @@
 """Differentiable Fock-like exchange and a Taylor-series TDKS propagator on the GPU.
 
-* ``FockApply`` is the autograd form of hse_fock_apply: forward runs the fused (complex64) or
-  staged (complex128) kernels, backward runs hse_fock_apply_vjp for the gradients with
+* ``FockApply`` is the autograd form of hse_fock_apply: forward runs the fused or (complex128,
+  larger grids) staged kernels, backward runs hse_fock_apply_vjp for the gradients with
   respect to the occupied orbitals, the target orbitals and omega.  Passing the same tensor
   as occupied and target set (the self-consistent case) gives the summed gradient.
 * ``KineticApply`` applies 1/2 |G + k + A|^2 (hse_kinetic_apply); the operator is Hermitian,
