@@ -933,6 +933,7 @@ __device__ __forceinline__ void pairconv_item(const PairArgs& args, int item, fl
   };
   if (it.q0 == it.q1) fold(true, false, true);  // no partners: zeros
   const int most = fold_terms(args.n_part, args.nk_part);
+  const int span = most / args.n_part;  // the same in whole k'
   int folds = 0, group = 0;  // folds so far; terms of the current group (MODE_OCC)
 
   // MODE_OCC with the omega gradient fused in: this slot's spectrum scratch and FP64 sum
@@ -985,7 +986,7 @@ __device__ __forceinline__ void pairconv_item(const PairArgs& args, int item, fl
       }
     }
     // the end of the item, or of a fold group: in the u_occ pass one that the next k' would overfill, in the
-    // others, which have no registers to count terms (24^3: 102.2 -> 102.6 ms), one of as many k'
+    // others, which have no registers to count terms (24^3: 102.3 -> 102.6 ms), one of as many k'
     const bool last = kp == kp_end - 1;
     if constexpr (MODE == MODE_OCC) {
       group += j1 - (kp == kp_begin ? j_begin : 0);
@@ -995,7 +996,7 @@ __device__ __forceinline__ void pairconv_item(const PairArgs& args, int item, fl
         group = 0;
       }
     } else {
-      const int span = most / args.n_part, grp = (kp - kp_begin) / span;
+      const int grp = (kp - kp_begin) / span;
       if (last || (kp - kp_begin + 1) % span == 0) fold(grp == 0, grp == 1, last);
     }
   }
